@@ -27,6 +27,7 @@
 #include "sg_sched.h"
 #include "sg_bits.cuh"
 #include "sg_stencil.cuh"
+#include "sg_words.cuh"
 
 namespace sg {
 
@@ -189,7 +190,7 @@ cudaError_t launch_batch(const sg_batch_plan *p, int parity, cudaStream_t st,
     }
 }
 
-// k fused steps of every gasket of the batch, bit-sliced (sg_bits.cuh): a
+// k fused steps of every gasket of a small batch, bit-sliced (sg_bits.cuh): a
 // warp takes one work item at a time, finds its gasket, decodes its tile at
 // that gasket's level and runs the k steps of the tile in shared memory.
 template <int S, int KH>
@@ -236,25 +237,148 @@ cudaError_t launch_batch_fused_t(const sg_batch_plan *p, int parity, int k, cuda
     return cudaGetLastError();
 }
 
+// k fused steps of every gasket of the batch, up to 32 tiles to a word
+// (sg_words.cuh).  The work list counts rho-tiles; each window of `window` of
+// its positions (a unit's worth) is two CTA jobs:
+//   * of the gaskets of level 9 or more, the units of 3^l 64-tiles whose first
+//     work item lies in the window;
+//   * the gaskets below level 9 (at most 9 64-tiles each) whose first work
+//     item lies in the window, as many at a time as 32 lanes hold: a lane's
+//     tile, its gasket, its buffers and its step count are the lane's own.
+constexpr int kSmallLevel = 8;
+
+__global__ void __launch_bounds__(kWordThreads, kWordCtas)
+ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k, int s, int l,
+                      uint32_t window)
+{
+    __shared__ uint32_t st[2][kWordBuf];
+    const uint32_t lane = threadIdx.x & 31u;
+    if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
+    const TripleRefs t = kTripleTable.t[threadIdx.x];
+    LambdaLane ll;
+    ll.init((int)lane, 0, order);
+    const uint32_t per = (uint32_t)pow3i(l + 6 - s);      // work items of a unit
+    const uint64_t windows = ((uint64_t)total + window - 1u) / window;
+    for (uint64_t job = blockIdx.x; job < 2u * windows; job += gridDim.x) {
+        const bool small = job >= windows;           // the units first, then the small gaskets
+        const uint64_t w0 = (small ? job - windows : job) * window;
+        const uint32_t begin = (uint32_t)w0;
+        const uint32_t end = (uint32_t)min(w0 + window, (uint64_t)total);
+        // 32 gaskets at a time from the one that holds the window's first item
+        for (uint32_t i0 = batch_instance(bv.prefix, bv.count, begin);; i0 += 32u) {
+            const uint32_t i = i0 + lane;
+            const bool have = i < bv.count;
+            const uint32_t first = have ? __ldg(bv.prefix + i) : ~0u;
+            const uint32_t next = have ? __ldg(bv.prefix + i + 1) : ~0u;
+            const int lv = have ? __ldg(bv.level + i) : 0;
+            const int r = lv & 0xFF, kk = (lv >> 8) ? (lv >> 8) : k;
+            const bool in_window = have && first < end;
+            // units of the large gaskets
+            uint32_t big = __ballot_sync(~0u, in_window && !small && r > kSmallLevel);
+            while (big != 0u) {
+                const int src = __ffs((int)big) - 1;
+                big &= big - 1u;
+                const int rg = __shfl_sync(~0u, r, src), kg = __shfl_sync(~0u, kk, src);
+                const uint32_t fg = __shfl_sync(~0u, first, src), ng = __shfl_sync(~0u, next, src);
+                const uint64_t pa = __ldg(bv.buf_a + i0 + src), pb = __ldg(bv.buf_b + i0 + src);
+                const uint8_t *in = reinterpret_cast<const uint8_t *>(parity ? pb : pa);
+                uint8_t *out = reinterpret_cast<uint8_t *>(parity ? pa : pb);
+                const int rbu = rg - 6 - l;
+                ll.set_level((int)lane, rbu);
+                const uint32_t W = pi_word(order, rbu);
+                uint32_t m = fg >= begin ? 0u : (begin - fg + per - 1u) / per;
+                for (; fg + m * per < min(end, ng); ++m) {
+                    const uint32_t hi = m / W, lo = m - hi * W;
+                    const uint2 c = ll.decode(lo, hi);
+                    const WordLane w = unit_lane(in, out, rg, l, c.x, c.y, lane);
+                    words_unit_steps(st, w, t, kg, kg, false);
+                }
+            }
+            // the small gaskets that begin in the window, packed into the lanes
+            bool todo = in_window && small && first >= begin && r <= kSmallLevel;
+            while (__any_sync(~0u, todo)) {
+                const int levels = max(r - 6, 0);
+                const uint32_t tiles = todo ? (uint32_t)pow3i(levels) : 0u;
+                uint32_t incl = tiles;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t v = __shfl_up_sync(~0u, incl, d);
+                    if ((int)lane >= d) incl += v;
+                }
+                const bool take = todo && incl <= 32u;
+                todo = todo && !take;
+                const uint32_t excl = incl - tiles;
+                // this lane's gasket: the taken one with excl <= lane < incl
+                int g = -1;
+                uint32_t taken = __ballot_sync(~0u, take);
+                int kmax = 0;
+                while (taken != 0u) {
+                    const int src = __ffs((int)taken) - 1;
+                    taken &= taken - 1u;
+                    const uint32_t e0 = __shfl_sync(~0u, excl, src), e1 = __shfl_sync(~0u, incl, src);
+                    kmax = max(kmax, __shfl_sync(~0u, kk, src));
+                    if (lane >= e0 && lane < e1) g = src;
+                }
+                const int gs = max(g, 0);
+                const int rg = __shfl_sync(~0u, r, gs), kg = __shfl_sync(~0u, kk, gs);
+                const uint32_t tile = lane - __shfl_sync(~0u, excl, gs);
+                WordLane w;
+                const uint64_t pa = __ldg(bv.buf_a + i0 + gs), pb = __ldg(bv.buf_b + i0 + gs);
+                w.in = reinterpret_cast<const uint8_t *>(parity ? pb : pa);
+                w.out = reinterpret_cast<uint8_t *>(parity ? pa : pb);
+                w.r = rg;
+                w.blocks = w.own = 0u;
+                w.x = w.y = w.ox = w.oy = 0u;
+                w.l = (uint32_t)max(rg - 6, 0);
+                w.nb = 1u << w.l;
+                w.base = lane - tile;
+                if (g >= 0) {
+                    const uint2 c = gasket_coords(tile, (int)w.l);
+                    const uint64_t at = ((uint64_t)(c.y << 6) << rg) + (c.x << 6);
+                    w.in += at;
+                    w.out += at;
+                    w.blocks = tile_blocks(rg);
+                    w.own = 1u;
+                    w.x = c.x;
+                    w.y = c.y;
+                }
+                words_unit_steps(st, w, t, g >= 0 ? kg : 0, kmax, true);
+            }
+            if (!__all_sync(~0u, in_window)) break;
+        }
+    }
+}
+
 // k steps (1 <= k <= SG_FUSE_MAX) of every gasket: one launch.
 cudaError_t launch_batch_k(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
                            const LaunchCfg &cfg)
 {
     if (k == 1) return launch_batch(p, parity, st, cfg);
     if (k < 1 || k > SG_FUSE_MAX) return cudaErrorInvalidValue;
-    const int kh = k <= 4 ? 4 : k <= 8 ? 8 : 16;
-    switch (p->rho * 100 + kh) {
-    case 1604: return launch_batch_fused_t<4, 4>(p, parity, k, st, cfg);
-    case 1608: return launch_batch_fused_t<4, 8>(p, parity, k, st, cfg);
-    case 1616: return launch_batch_fused_t<4, 16>(p, parity, k, st, cfg);
-    case 3204: return launch_batch_fused_t<5, 4>(p, parity, k, st, cfg);
-    case 3208: return launch_batch_fused_t<5, 8>(p, parity, k, st, cfg);
-    case 3216: return launch_batch_fused_t<5, 16>(p, parity, k, st, cfg);
-    case 6404: return launch_batch_fused_t<6, 4>(p, parity, k, st, cfg);
-    case 6408: return launch_batch_fused_t<6, 8>(p, parity, k, st, cfg);
-    case 6416: return launch_batch_fused_t<6, 16>(p, parity, k, st, cfg);
-    default: return cudaErrorInvalidValue;
+    const int s = p->rho == 16 ? 4 : p->rho == 32 ? 5 : 6;
+    // Few tiles: a warp per 16- or 32-tile is the shorter chain, by the same
+    // lines as for one gasket (launch_ca_fused in sg_fused.cu, in cells)
+    const uint64_t cells = (uint64_t)p->total_tiles * (uint64_t)pow3i(s);
+    if (s == 4 && (cells <= (uint64_t)pow3i(10) || (cells <= (uint64_t)pow3i(11) && k <= 8))) {
+        if (k <= 4) return launch_batch_fused_t<4, 4>(p, parity, k, st, cfg);
+        if (k <= 8) return launch_batch_fused_t<4, 8>(p, parity, k, st, cfg);
+        return launch_batch_fused_t<4, 16>(p, parity, k, st, cfg);
     }
+    if (s == 5 && cells <= (uint64_t)pow3i(12) && k <= 8) {
+        if (k <= 4) return launch_batch_fused_t<5, 4>(p, parity, k, st, cfg);
+        return launch_batch_fused_t<5, 8>(p, parity, k, st, cfg);
+    }
+    static std::atomic<int> occ{0};
+    const int l = cells >= (uint64_t)pow3i(13) ? 3 : 2;
+    const uint32_t window = (uint32_t)pow3i(l + 6 - s);
+    unsigned grid = 1;
+    cudaError_t e = persistent_grid(ca_batch_words_kernel, kWordThreads, 0,
+                                    2u * (((uint64_t)p->total_tiles + window - 1) / window), cfg,
+                                    &grid, &occ);
+    if (e != cudaSuccess) return e;
+    ca_batch_words_kernel<<<grid, kWordThreads, 0, st>>>(view_of(p), p->total_tiles, parity,
+                                                         cfg.order, k, s, l, window);
+    return cudaGetLastError();
 }
 
 bool plan_ok(const sg_batch_plan *p)

@@ -16,7 +16,9 @@
 //     and produce zeros at every step, exactly as the single-step kernels
 //     treat them (off-gasket cells are 0 in every state).
 //
-// The CA runs bit-sliced (one warp per tile, 32 cells per word operation).
+// The CA runs bit-sliced: one warp per tile on rows of bits (32 cells per word
+// operation), and under lambda on large gaskets one bit per tile, 32 tiles per
+// word operation (sg_words.cuh).
 // Diffusion at tile sides 32 and 64 runs one warp per 32 x 32 unit with the
 // 9-cell gasket blocks of 4 x 4 cells held in registers (diffuse_warp_fused_
 // kernel, below); at side 16 one CTA per tile on float4 chunks
@@ -29,6 +31,7 @@
 #include "sg_bits.cuh"
 #include "sg_stencil.cuh"
 #include "sg_tma.cuh"
+#include "sg_words.cuh"
 
 namespace sg {
 
@@ -508,6 +511,53 @@ diffuse_warp_fused_kernel(const float *__restrict__ in, float *__restrict__ out,
 }
 
 // ---------------------------------------------------------------------------
+// CA under lambda on large gaskets: units of up to 27 64-tiles, one bit per tile
+// (sg_words.cuh), whatever tile side was asked for -- it names launch
+// geometry, not results.  One CTA per unit.
+//
+// Bound: the DRAM pattern of the touched sectors (60 MB in, 60 MB out at level
+// 15), which 32-byte scattered stores sustain at about 3.3 TB/s whatever the
+// kernel; the steps add 0.45 us each.  Level 15, 16 steps: 153.7 us with dense
+// bit rows, 45.0 us here (2 steps: 59.4 and 38.6; level 14, 16 steps: 54.5 and
+// 13.6).  Three CTAs an SM (80 registers, the loads of a unit all in flight)
+// beat five (48 registers, with spills): 45.0 against 47.3 us.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kWordThreads, kWordCtas)
+ca_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
+                int l, uint32_t units, int k)
+{
+    __shared__ uint32_t st[2][kWordBuf];
+    const uint32_t lane = threadIdx.x & 31u;
+    if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
+    const TripleRefs t = kTripleTable.t[threadIdx.x];
+    const int rbu = r > 6 ? r - 6 - l : 0;
+    LambdaLane ll;
+    ll.init((int)lane, rbu, order);
+    const uint32_t W = pi_word(order, rbu);
+    for (uint32_t q = blockIdx.x; q < units; q += gridDim.x) {
+        const uint2 c = decode_tile<kMapLambda>(q, units, rbu, W, ll);
+        const WordLane w = unit_lane(in, out, r, l, c.x, c.y, lane);
+        words_unit_steps(st, w, t, k, k, r < 6);
+    }
+}
+
+cudaError_t launch_ca_words(int r, const uint8_t *in, uint8_t *out, int k, cudaStream_t st,
+                            const LaunchCfg &cfg)
+{
+    static std::atomic<int> occ{0};
+    // 27 tiles a unit fill the word (2 and 16 steps at level 13: 6.9 and 9.4 us,
+    // against 7.1 and 10.2 with 9 tiles); below, 9 tiles spread a launch over
+    // more SMs (level 12: 5.6 and 8.1 us against 6.9 and 9.3)
+    const int l = min(r >= 13 ? 3 : 2, max(r - 6, 0));
+    const uint32_t units = (uint32_t)pow3i(r > 6 ? r - 6 - l : 0);
+    unsigned grid = 1;
+    cudaError_t e = persistent_grid(ca_words_kernel, kWordThreads, 0, units, cfg, &grid, &occ);
+    if (e != cudaSuccess) return e;
+    ca_words_kernel<<<grid, kWordThreads, 0, st>>>(in, out, r, cfg.order, l, units, k);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
 template <int S, int KH, int MAP>
@@ -605,9 +655,21 @@ cudaError_t launch_ca_fused(int r, int s, int map, const uint8_t *in, uint8_t *o
         SG_FUSED_SWITCH(s, k, CALL);
 #undef CALL
     }
-#define CALL(S, KH) launch_ca_fused_t<S, KH, kMapLambda>(r, in, out, k, st, cfg)
-    SG_FUSED_SWITCH(s, k, CALL);
-#undef CALL
+    // Small gaskets leave the chip to one wave of warps whichever kernel runs:
+    // there a warp per small tile is the shorter chain.  us for 2 / 8 / 16 steps,
+    // dense bit rows on 16-tiles (level 12: 32-tiles) against words: level 9,
+    // 2.8 / 4.2 / 7.1 and 5.2 / 6.2 / 8.1; level 11, 3.4 / 5.4 / 8.9 and 5.4 / 6.7 /
+    // 8.1; level 12, 4.2 / 6.5 / 12.6 and 5.6 / 6.6 / 8.1.
+    if (r <= 10 || (r == 11 && k <= 8)) {
+        if (k <= 4) return launch_ca_fused_t<4, 4, kMapLambda>(r, in, out, k, st, cfg);
+        if (k <= 8) return launch_ca_fused_t<4, 8, kMapLambda>(r, in, out, k, st, cfg);
+        return launch_ca_fused_t<4, 16, kMapLambda>(r, in, out, k, st, cfg);
+    }
+    if (r == 12 && k <= 8) {
+        if (k <= 4) return launch_ca_fused_t<5, 4, kMapLambda>(r, in, out, k, st, cfg);
+        return launch_ca_fused_t<5, 8, kMapLambda>(r, in, out, k, st, cfg);
+    }
+    return launch_ca_words(r, in, out, k, st, cfg);
 }
 
 cudaError_t launch_diffuse_fused(int r, int s, int map, const float *in, float *out,
