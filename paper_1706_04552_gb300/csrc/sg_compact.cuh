@@ -288,8 +288,8 @@ cudaError_t launch_compact_ca(int r, int s, int order, const uint8_t *in, uint8_
                               cudaStream_t st, const LaunchCfg &cfg);
 cudaError_t launch_compact_diffuse(int r, int s, int order, const float *in, float *out,
                                    float alpha, cudaStream_t st, const LaunchCfg &cfg);
-// k (2 .. SG_FUSE_MAX) CA steps in one launch, rho = 64 (sg_compact_fused.cu).
-cudaError_t launch_compact_ca_fused(int r, int order, const uint8_t *in, uint8_t *out, int k,
+// k (1 .. SG_FUSE_MAX) CA steps in one launch, rho = 64 (sg_compact_fused.cu).
+cudaError_t launch_compact_ca_words(int r, int order, const uint8_t *in, uint8_t *out, int k,
                                     cudaStream_t st, const LaunchCfg &cfg);
 
 }  // namespace sg

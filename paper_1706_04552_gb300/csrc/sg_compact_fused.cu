@@ -1,202 +1,161 @@
-// sg_compact_fused.cu -- k B3/S23 steps per launch on a compact array of
-// 64-tiles (layout in sg_compact.cuh), k <= SG_FUSE_MAX.
+// sg_compact_fused.cu -- B3/S23 steps on a compact array of 64-tiles (layout in
+// sg_compact.cuh), k <= SG_FUSE_MAX per launch, on words of 32 tiles.
 //
-// One warp takes one tile at a time and runs the bit-sliced k-step routine
-// of the embedded fused CA (bits_ca_step in sg_bits.cuh) on it: rows of
-// bits with a halo of KH rows above and below and 16 columns either side.
-// What differs is the staging.  The halo cells live in the compact runs of
-// the neighbouring tiles, and a KH-step light cone reaches only part of
-// them: the rows 64-KH .. 63 of the tiles above, the rows 0 .. KH-1 of the
-// tiles below, and of the tile to the left only its rows 0 .. 15 (its
-// columns 48 .. 63 hold gasket cells nowhere else).  Those runs are read as
-// whole sectors and packed to bits by ballots; each staged 16-column chunk
-// then takes its cells from them (a chunk's cells are consecutive in compact
-// order) and spreads them onto its columns through the row codec.  The tile
-// rows are gathered back to compact order at the end.
-#include "sg_bits.cuh"
+// The steps are those of sg_words.cuh: a unit is up to 27 64-tiles of one block
+// and the three tiles at its corners, one bit per tile, whatever order the
+// tiles have in memory (lambda_index gives each lane its tile's place).  What
+// differs is the way in and out.  A tile is a run of 729 bytes at any byte
+// address; lane t reads its own tile's run in aligned 16-byte pieces, packs
+// each to 16 bits, shifts the bits to the run's start, and a 32 x 32 bit
+// transpose across the warp turns "32 cells of my tile" into "my cell of 32
+// tiles".  On the way out the bits are shifted to the alignment of the output
+// run, and only its first and last pieces, shared with the neighbouring runs,
+// are stored byte by byte.
+//
+// Bound: latency and issue, half and half (the state stays in L2: 14.3 MB read
+// and written at level 15).  Level 15, 16 steps: 180.0 us with dense rows of
+// bits and a 16-cell halo, 24.5 here; level 10: 26.4 and 9.5.
 #include "sg_compact.cuh"
+#include "sg_words.cuh"
 
 namespace sg {
 
 namespace {
 
-// The neighbour tiles s = 0 .. 8, (dtx, dty) = (s % 3 - 1, s / 3 - 1), and
-// the compact elements [lo[s], hi[s]) of each that a KH-step light cone
-// reaches; staged as bits from word word[s] on, each run padded to whole
-// words.
-template <int KH> struct HaloRuns {
-    uint16_t lo[9], hi[9], word[9];
-    int words;
+// Word of the e-th cell of a tile (rows top to bottom, each left to right);
+// the positions past the last cell have none.
+struct CellTable {
+    uint16_t at[736];
 };
-
-template <int KH> constexpr HaloRuns<KH> make_halo_runs()
+constexpr CellTable make_cell_table()
 {
-    const RowCodec rc = make_row_codec();
-    auto start = [&](int y) { return y >= 64 ? kUnit : (int)rc.row_start[y]; };
-    HaloRuns<KH> h{};
-    int w = 0;
-    for (int s = 0; s < 9; ++s) {
-        const int dtx = s % 3 - 1, dty = s / 3 - 1;
-        int y0 = dty < 0 ? 64 - KH : 0, y1 = dty > 0 ? KH : 64;
-        if (dtx < 0 && y1 > 16) y1 = 16;       // left: columns 48..63 only in rows 0..15
-        if (y1 < y0) y1 = y0;
-        h.lo[s] = (uint16_t)start(y0);
-        h.hi[s] = (uint16_t)start(y1);
-        h.word[s] = (uint16_t)w;
-        w += (h.hi[s] - h.lo[s] + 31) / 32;
+    CellTable t{};
+    int e = 0;
+    for (uint32_t y = 0; y < 64u; ++y)
+        for (uint32_t x = 0; x < 64u; ++x)
+            if ((x & y) == 0u)
+                t.at[e++] = (uint16_t)(((y & 1u) ? 2u : (x & 1u)) * kPlane +
+                                       gasket_digits(x >> 1, y >> 1, 5));
+    for (; e < 736; ++e) t.at[e] = kNoWord;
+    return t;
+}
+__device__ const CellTable kCellTable = make_cell_table();
+
+// 16 bytes at p (16-byte aligned) as 16 bits.  Bytes outside [lo, hi) -- the
+// whole array -- are not read and give 0.
+__device__ __forceinline__ uint32_t piece_bits(const uint8_t *p, const uint8_t *lo,
+                                               const uint8_t *hi)
+{
+    if (p >= lo && p + 16 <= hi) {
+        const uint4 c = __ldg(reinterpret_cast<const uint4 *>(p));
+        return add_nibble(add_nibble(add_nibble(add_nibble(0u, c.w), c.z), c.y), c.x);
     }
-    h.words = w;
-    return h;
+    uint32_t v = 0u;
+#pragma unroll 1
+    for (int i = 0; i < 16; ++i)
+        if (p + i >= lo && p + i < hi) v |= (uint32_t)(p[i] & 1u) << i;
+    return v;
 }
 
-template <int KH> struct HaloRunWords {
-    static constexpr int value = make_halo_runs<KH>().words;
-};
-
-__device__ const HaloRuns<4> kHaloRuns4 = make_halo_runs<4>();
-__device__ const HaloRuns<8> kHaloRuns8 = make_halo_runs<8>();
-__device__ const HaloRuns<16> kHaloRuns16 = make_halo_runs<16>();
-
-template <int KH> __device__ __forceinline__ const HaloRuns<KH> &halo_runs()
+// Cells 96 W .. 96 W + 95 of every lane's tile -> words (warp W).
+__device__ __forceinline__ void run_to_words(uint32_t *s, const uint8_t *run, bool on,
+                                             const uint8_t *lo, const uint8_t *hi,
+                                             const Transpose &tr, int warp, int lane)
 {
-    if constexpr (KH == 4) return kHaloRuns4;
-    else if constexpr (KH == 8) return kHaloRuns8;
-    else return kHaloRuns16;
+    const uint32_t off = (uint32_t)((uintptr_t)run & 15u);
+    const uint8_t *p = run - off + 96 * warp;
+    uint32_t b[4] = {0u, 0u, 0u, 0u};                 // 7 pieces: 112 bits from the aligned start
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const bool some = on && 96 * warp + 16 * i < (int)off + kUnit;
+        if (some) b[i >> 1] |= piece_bits(p + 16 * i, lo, hi) << (16 * (i & 1));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int g = 3 * warp + i;
+        if (g > 22) break;
+        const uint32_t x = tr(__funnelshift_r(b[i], b[i + 1], off));
+        const uint32_t a = kCellTable.at[32 * g + lane];
+        if (a != kNoWord) s[a] = x;
+    }
 }
 
-template <int KH>
-__global__ void __launch_bounds__(kUnitThreads, 6)
-compact_ca_fused_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r,
-                        int order, uint32_t total, int k)
+// The pieces 6 W .. 6 W + 5 of every own tile's output run.
+__device__ __forceinline__ void words_to_run(const uint32_t *s, uint8_t *run, bool own,
+                                             const Transpose &tr, int warp, int lane)
 {
-    constexpr int S = 6;
-    using B = BitShape<S, KH>;
-    constexpr int HPR = 2 * B::WPR;
-    constexpr int RUN_WORDS = HaloRunWords<KH>::value;
-    constexpr int OUT_WORDS = (kUnit + 31) / 32;
-    __shared__ RowCodec tc;
-    __shared__ uint32_t sm[kUnitWarps][3][B::BUFW];           // two states and the mask
-    __shared__ uint32_t runs[kUnitWarps][RUN_WORDS + 2];      // + guard words
-    __shared__ uint32_t obits[kUnitWarps][OUT_WORDS + 3];
-    {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(&kRowCodec);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&tc);
-        for (int i = threadIdx.x; i < (int)(sizeof(RowCodec) / 4); i += kUnitThreads)
-            dst[i] = src[i];
+    uint32_t g[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int e = 96 * warp - 32 + 32 * i + lane;
+        const uint32_t a = e >= 0 && e < 736 ? kCellTable.at[e] : kNoWord;
+        g[i] = tr(a != kNoWord ? s[a] : 0u);
     }
+    if (!own) return;
+    const uint32_t off = (uint32_t)((uintptr_t)run & 15u);
+    uint8_t *p = run - off + 96 * warp;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        uint32_t v = __funnelshift_l(g[i], g[i + 1], off);
+#pragma unroll
+        for (int h = 0; h < 2; ++h, v >>= 16) {
+            const int e = 96 * warp + 32 * i + 16 * h - (int)off;      // first cell of the piece
+            uint8_t *q = p + 32 * i + 16 * h;
+            if (e >= 0 && e + 16 <= kUnit) {
+                *reinterpret_cast<uint4 *>(q) = make_uint4(nibble_bytes(v, 0), nibble_bytes(v, 1),
+                                                           nibble_bytes(v, 2), nibble_bytes(v, 3));
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < 16; ++j)
+                    if (e + j >= 0 && e + j < kUnit) q[j] = (uint8_t)((v >> j) & 1u);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kWordThreads, kWordCtas)
+compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
+                     int l, uint32_t units, uint32_t total, int k)
+{
+    __shared__ uint32_t st[2][kWordBuf];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t *st0 = sm[warp][0] + 1, *st1 = sm[warp][1] + 1, *mk = sm[warp][2] + 1;
-    uint32_t *cb = runs[warp], *ob = obits[warp];
-    if (lane < 2) cb[RUN_WORDS + lane] = 0u;
-    __syncthreads();
-
-    const HaloRuns<KH> &hr = halo_runs<KH>();
-    const int rb = r - S;
-    const int n = 1 << r;
-    const uint32_t units = total / kUnit;                     // whole tiles: r >= 6
+    if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
+    const TripleRefs t = kTripleTable.t[threadIdx.x];
+    Transpose tr;
+    const int rbu = r - 6 - l;
     LambdaLane ll;
-    ll.init(lane, rb, order);
-    const uint32_t W = pi_word(order, rb);
-    const uint32_t nwarps = gridDim.x * kUnitWarps;
-    for (uint32_t u = blockIdx.x * kUnitWarps + warp; u < units; u += nwarps) {
-        const uint32_t bq = u / W, aq = u - bq * W;
-        const uint2 b = ll.decode(aq, bq);
-        // launch index of neighbour tile `lane` (lanes 0..8), ~0u if it has
-        // no gasket cell or lies outside the grid
-        uint32_t nq = ~0u;
-        if (lane < 9) {
-            const uint32_t nbx = b.x + (uint32_t)(lane % 3 - 1), nby = b.y + (uint32_t)(lane / 3 - 1);
-            if ((nbx >> rb) == 0u && (nby >> rb) == 0u && (nbx & nby) == 0u)
-                nq = lambda_index(nbx, nby, rb, order);
-        }
-        __syncwarp();                  // the previous tile is finished with the buffers
-        // 1. the runs as bits (whole sectors, then ballots)
-        for (int s = 0; s < 9; ++s) {
-            const uint32_t q = __shfl_sync(0xffffffffu, nq, s);
-            const int lo = hr.lo[s], hi = hr.hi[s], w0 = hr.word[s];
-            for (int e = lo; e < hi; e += 32) {
-                const int c = e + lane;
-                const uint8_t v = (q != ~0u && c < hi) ? in[(uint64_t)q * kUnit + c] : 0;
-                const uint32_t w = __ballot_sync(0xffffffffu, v != 0);
-                if (lane == 0) cb[w0 + (e - lo) / 32] = w;
-            }
-        }
-        __syncwarp();
-        // 2. staged rows: each 16-column chunk from its tile's run
-        const int x0 = (int)(b.x << S), y0 = (int)(b.y << S);
-        uint16_t *bh = reinterpret_cast<uint16_t *>(st0);
-        uint16_t *mh = reinterpret_cast<uint16_t *>(mk);
-        for (int i = lane; i < B::ROWS * HPR; i += 32) {
-            const int row = i / HPR, h = i - row * HPR;
-            const int x = x0 - 16 + 16 * h, y = y0 - KH + row;
-            uint32_t v = 0u, m = 0u;
-            if (h < B::HW && x >= 0 && y >= 0 && x < n && y < n && (x & y) == 0) {
-                const int s = ((y >> S) - y0 / 64 + 1) * 3 + ((x >> S) - x0 / 64 + 1);
-                const uint32_t lx = (uint32_t)x & 63u, ly = (uint32_t)y & 63u;
-                const uint32_t cx = lx >> 4, n16 = 16u >> __popc(ly & 15u);
-                const uint32_t rank = __popc(member_bits4(ly >> 4) & ((1u << cx) - 1u));
-                const uint32_t e = tc.row_start[ly] + rank * n16;
-                const uint32_t o = (uint32_t)hr.word[s] * 32u + (e - hr.lo[s]);
-                const uint32_t bits = __funnelshift_r(cb[o >> 5], cb[(o >> 5) + 1], o & 31u);
-                const uint32_t yl = ly & 7u, n8 = 8u >> __popc(yl), m8 = (1u << n8) - 1u;
-                v = tc.dep[yl][bits & m8];
-                if ((ly & 8u) == 0u) v |= (uint32_t)tc.dep[yl][(bits >> n8) & m8] << 8;
-                m = member_bits16(ly & 15u);
-            }
-            bh[i] = (uint16_t)v;
-            mh[i] = (uint16_t)m;
-        }
-        if (lane < OUT_WORDS + 3) ob[lane] = 0u;
-        __syncwarp();
-        // 3. k steps in shared memory
-        for (int step = 1; step <= k; ++step) {
-            bits_ca_step<S, KH>((step & 1) ? st0 : st1, (step & 1) ? st1 : st0, mk, step, lane);
-            __syncwarp();
-        }
-        // 4. tile rows back to compact order, then bytes
-        const uint32_t *fin = (k & 1) ? st1 : st0;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const uint32_t ty = 2u * lane + j;
-            const uint32_t *p = fin + (KH + ty) * B::WPR;   // columns -16 .. 79
-            const uint64_t row = (uint64_t)__funnelshift_r(p[0], p[1], 16) |
-                                 ((uint64_t)__funnelshift_r(p[1], p[2], 16) << 32);
-            or_bits_at(ob, tc.row_start[ty], gather_row(tc, row, ty));
-        }
-        __syncwarp();
-        const uint32_t base = u * kUnit;
-#pragma unroll
-        for (int it = 0; it < OUT_WORDS; ++it) {
-            const int c = 32 * it + lane;
-            if (c < kUnit) out[base + c] = (uint8_t)((ob[it] >> lane) & 1u);
-        }
+    ll.init(lane, rbu, order);
+    const uint32_t W = pi_word(order, rbu);
+    for (uint32_t q = blockIdx.x; q < units; q += gridDim.x) {
+        const uint2 c = decode_tile<kMapLambda>(q, units, rbu, W, ll);
+        const WordLane w = unit_lane(nullptr, nullptr, r, l, c.x, c.y, (uint32_t)lane);
+        const bool on = w.blocks != 0u;
+        const uint64_t at = (uint64_t)lambda_index(w.x, w.y, r - 6, order) * kUnit;
+        tr.init(lane);
+        run_to_words(st[k & 1], in + at, on, in, in + total, tr, warp, lane);
+        words_steps(st, w, t, k, k, false);
+        tr.init(lane);
+        words_to_run(st[0], out + at, w.own, tr, warp, lane);
+        __syncthreads();                 // the words are read before the next unit's are written
     }
-}
-
-template <int KH>
-cudaError_t launch_fused_t(int r, int order, const uint8_t *in, uint8_t *out, int k,
-                           cudaStream_t st, const LaunchCfg &cfg)
-{
-    static std::atomic<int> occ{0};
-    const uint32_t total = (uint32_t)pow3i(r);
-    const uint64_t units = total / kUnit;
-    unsigned grid = 1;
-    auto kern = compact_ca_fused_kernel<KH>;
-    cudaError_t e = persistent_grid(kern, kUnitThreads, 0, (units + kUnitWarps - 1) / kUnitWarps,
-                                    cfg, &grid, &occ);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, kUnitThreads, 0, st>>>(in, out, r, order, total, k);
-    return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_compact_ca_fused(int r, int order, const uint8_t *in, uint8_t *out, int k,
+cudaError_t launch_compact_ca_words(int r, int order, const uint8_t *in, uint8_t *out, int k,
                                     cudaStream_t st, const LaunchCfg &cfg)
 {
-    if (k <= 4) return launch_fused_t<4>(r, order, in, out, k, st, cfg);
-    if (k <= 8) return launch_fused_t<8>(r, order, in, out, k, st, cfg);
-    return launch_fused_t<16>(r, order, in, out, k, st, cfg);
+    static std::atomic<int> occ{0};
+    // unit depth as for the embedded kernel (16 steps, 9 against 27 tiles: level
+    // 12, 9.5 and 10.0 us; level 13, 10.3 and 9.9; level 14, 20.4 and 11.8)
+    const int l = min(r >= 13 ? 3 : 2, r - 6);
+    const uint32_t units = (uint32_t)pow3i(r - 6 - l);
+    unsigned grid = 1;
+    cudaError_t e = persistent_grid(compact_words_kernel, kWordThreads, 0, units, cfg, &grid, &occ);
+    if (e != cudaSuccess) return e;
+    compact_words_kernel<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units,
+                                                        (uint32_t)pow3i(r), k);
+    return cudaGetLastError();
 }
 
 }  // namespace sg

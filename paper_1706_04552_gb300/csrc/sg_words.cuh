@@ -479,19 +479,16 @@ __device__ __forceinline__ uint32_t maj3w(uint32_t a, uint32_t b, uint32_t c)
     return (a & b) | (c & (a ^ b));
 }
 
-// k steps of the unit's tiles: every thread of the CTA (kWordThreads) calls it
-// with its lane's tile.  st: two buffers whose words kWordZero are 0.  kk:
-// this lane's step count, k the largest; mixed: some lane's count differs or
-// some lane's grid fills only part of its tile (its other cells stay 0).
-__device__ __forceinline__ void words_unit_steps(uint32_t (&st)[2][kWordBuf], const WordLane &w,
-                                                 const TripleRefs &t, int kk, int k, bool mixed)
+// k steps on the words in st[k & 1], written by the CTA's warps just before
+// (the call begins with a barrier); the result is in st[0], behind a barrier.
+// Every thread of the CTA (kWordThreads) calls it with its lane's tile.  st:
+// two buffers whose words kWordZero are 0.  kk: this lane's step count, k the
+// largest; mixed: some lane's count differs or some lane's grid fills only
+// part of its tile (its other cells stay 0).
+__device__ __forceinline__ void words_steps(uint32_t (&st)[2][kWordBuf], const WordLane &w,
+                                            const TripleRefs &t, int kk, int k, bool mixed)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    Transpose tr;
-    tr.init(lane);
-#define CALL(Q, U) group_to_words<Q>(st[k & 1], w, U, tr, lane)
-    SG_WORD_PIECES(CALL);
-#undef CALL
     // the last warp's lanes pass the corner words between the bits: the bit
     // they take from a corner's B or C cell, or A cell, and their own kinds
     uint32_t fa1 = 0u, fa2 = 0u, fb1 = 0u, fb2 = 0u, fc1 = 0u, fc2 = 0u, ml = 0u, mu = 0u;
@@ -565,6 +562,19 @@ __device__ __forceinline__ void words_unit_steps(uint32_t (&st)[2][kWordBuf], co
         if (s >= 0) step(st[0], st[1], s);
         step(st[1], st[0], s + 1);
     }
+}
+
+// k steps of a unit of embedded tiles: rows to words, steps, words to rows.
+__device__ __forceinline__ void words_unit_steps(uint32_t (&st)[2][kWordBuf], const WordLane &w,
+                                                 const TripleRefs &t, int kk, int k, bool mixed)
+{
+    const int lane = threadIdx.x & 31;
+    Transpose tr;
+    tr.init(lane);
+#define CALL(Q, U) group_to_words<Q>(st[k & 1], w, U, tr, lane)
+    SG_WORD_PIECES(CALL);
+#undef CALL
+    words_steps(st, w, t, kk, k, mixed);
     // 32-byte stores where every tile's address allows them (16-byte ones halve
     // the sectors a request carries: 38.7 against 42.8 us at level 15, k = 2)
     const bool wide = __all_sync(~0u, !w.own || (w.r > 4 && ((uintptr_t)w.out & 31u) == 0u));

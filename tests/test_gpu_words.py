@@ -79,3 +79,49 @@ def test_scheduler_mixes_step_counts_in_a_word():
         assert np.array_equal(cur.cpu().numpy().reshape(n, n),
                               oracle.ca_steps(levels[i], host[i], steps[i])), i
     sched.close()
+
+
+@pytest.mark.parametrize("r,k,order,shift_in,shift_out", [
+    (6, 1, "interleaved", 0, 0), (6, 16, "interleaved", 5, 11), (7, 3, "rowmajor", 15, 0),
+    (8, 16, "rowmajor", 0, 1), (9, 2, "interleaved", 1, 15), (10, 16, "interleaved", 3, 8),
+    (12, 16, "rowmajor", 0, 0), (13, 7, "interleaved", 0, 4),
+])
+def test_compact_steps_at_any_alignment(r, k, order, shift_in, shift_out):
+    n, c = 1 << r, 3 ** r
+    oid = {"rowmajor": oracle.ORDER_ROWMAJOR, "interleaved": oracle.ORDER_INTERLEAVED}[order]
+    s0 = _state(r, 50 + r)
+    src = torch.full((c + 64,), 1, dtype=torch.uint8, device="cuda")
+    dst = torch.full((c + 64,), 7, dtype=torch.uint8, device="cuda")
+    a, b = src[shift_in:shift_in + c], dst[shift_out:shift_out + c]
+    a.copy_(torch.from_numpy(oracle.compact_pack(r, 6, s0, oid)))
+    sg.compact_ca_steps(a, b, r, 64, k, order=order)
+    want = oracle.compact_pack(r, 6, oracle.ca_steps(r, s0, k), oid)
+    got = dst.cpu().numpy()
+    assert np.array_equal(got[shift_out:shift_out + c], want)
+    assert (got[:shift_out] == 7).all() and (got[shift_out + c:] == 7).all()
+
+
+def test_single_steps_on_words_match_the_general_path():
+    # level 14 is the smallest a single step takes on words (embedded, compact
+    # and batched); the bounding-box map runs the general tile kernel
+    r = 14
+    n = 1 << r
+    idx, val = inputs.ca_seed_sparse(r, 0.4, 5)
+    a = torch.zeros(n * n, dtype=torch.uint8, device="cuda")
+    a[torch.from_numpy(idx).cuda()] = torch.from_numpy(val).cuda()
+    want, got = torch.zeros_like(a), torch.zeros_like(a)
+    sg.ca_step(a, want, r, 64, "bbox")
+    for rho in (4, 64):
+        got.zero_()
+        sg.ca_step(a, got, r, rho)
+        assert torch.equal(got, want)
+    c, d, e = (torch.zeros(3 ** r, dtype=torch.uint8, device="cuda") for _ in range(3))
+    sg.compact_pack(a, c, r, 64)
+    sg.compact_ca_step(c, d, r, 64)
+    sg.compact_pack(want, e, r, 64)
+    assert torch.equal(d, e)
+    small = torch.from_numpy(_state(7, 1).ravel()).cuda()
+    sa, sb = [small, a], [torch.zeros_like(small), torch.zeros_like(a)]
+    sg.CABatch([7, r], sa, sb, rho=32).step(0)
+    assert torch.equal(sb[1], want)
+    assert np.array_equal(sb[0].cpu().numpy().reshape(128, 128), oracle.ca_steps(7, _state(7, 1), 1))

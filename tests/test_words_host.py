@@ -127,3 +127,40 @@ def test_words_match_the_oracle(r, depth, k):
                     xx, yy = bx * 64 + 2 * x + dx, by * 64 + 2 * y + dy
                     inside = xx < n and yy < n
                     assert w[c, p, t] == (want[yy, xx] if inside else 0)
+
+
+@pytest.mark.parametrize("off_in,off_out", [(0, 0), (1, 15), (7, 3), (8, 8), (15, 1)])
+def test_compact_runs_shift_to_any_alignment(off_in, off_out):
+    # a 729-byte run read in aligned 16-byte pieces: cells 96 W + 32 i .. + 31 of
+    # warp W come from a funnel shift of its pieces' bits; the way out shifts
+    # the same groups to the output's alignment
+    cells = np.random.default_rng(off_in).integers(0, 2, 729)
+    flat = np.concatenate([np.ones(off_in, int), cells, np.ones(64, int)])   # neighbours around
+    groups = {}
+    for warp in range(8):
+        b = [0, 0, 0, 0]
+        for i in range(7):
+            start = 96 * warp + 16 * i
+            if start < off_in + 729:
+                v = sum(int(x) << j for j, x in enumerate(flat[start:start + 16]))
+                b[i >> 1] |= v << (16 * (i & 1))
+        for i in range(3):
+            if 3 * warp + i <= 22:
+                x = ((b[i] | b[i + 1] << 32) >> off_in) & 0xFFFFFFFF
+                groups[3 * warp + i] = x
+    for e in range(729):
+        assert (groups[e >> 5] >> (e & 31)) & 1 == cells[e]
+    valid = {g: v if g < 22 else v & ((1 << 25) - 1) for g, v in groups.items()}
+    out = np.full(off_out + 729 + 64, -1)
+    for warp in range(8):
+        g = [valid.get(3 * warp - 1 + i, 0) for i in range(4)]
+        for i in range(3):
+            v = (((g[i + 1] << 32 | g[i]) << off_out) >> 32) & 0xFFFFFFFF
+            for h in range(2):
+                first = 96 * warp + 32 * i + 16 * h - off_out
+                for j in range(16):
+                    if 0 <= first + j < 729:
+                        assert out[off_out + first + j] == -1          # stored once
+                        out[off_out + first + j] = (v >> (16 * h + j)) & 1
+    assert np.array_equal(out[off_out:off_out + 729], cells)
+    assert (out[:off_out] == -1).all() and (out[off_out + 729:] == -1).all()
