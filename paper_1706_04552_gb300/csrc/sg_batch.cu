@@ -247,9 +247,25 @@ cudaError_t launch_batch_fused_t(const sg_batch_plan *p, int parity, int k, cuda
 //     tile, its gasket, its buffers and its step count are the lane's own.
 constexpr int kSmallLevel = 8;
 
+// batch_instance by a whole warp: 32 probes at a time, so that the search costs
+// one memory latency per factor of 32 (every lane passes the same q).
+__device__ __forceinline__ uint32_t batch_instance_warp(const uint32_t *prefix, uint32_t count,
+                                                        uint32_t q, uint32_t lane)
+{
+    uint32_t lo = 0, n = count;                        // prefix[lo] <= q < prefix[lo + n]
+    while (n > 1u) {
+        const uint32_t step = (n + 31u) / 32u, at = lane * step;
+        const uint32_t hit = __ballot_sync(~0u, at < n && __ldg(prefix + lo + at) <= q);
+        const uint32_t skip = (31u - (uint32_t)__clz((int)hit)) * step;   // lane 0 always hits
+        lo += skip;
+        n = min(step, n - skip);
+    }
+    return lo;
+}
+
 __global__ void __launch_bounds__(kWordThreads, kWordCtas)
 ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k, int s, int l,
-                      uint32_t window)
+                      uint32_t window, bool any_small)
 {
     __shared__ uint32_t st[2][kWordBuf];
     const uint32_t lane = threadIdx.x & 31u;
@@ -259,18 +275,20 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
     ll.init((int)lane, 0, order);
     const uint32_t per = (uint32_t)pow3i(l + 6 - s);      // work items of a unit
     const uint64_t windows = ((uint64_t)total + window - 1u) / window;
-    for (uint64_t job = blockIdx.x; job < 2u * windows; job += gridDim.x) {
+    for (uint64_t job = blockIdx.x; job < (any_small ? 2u : 1u) * windows; job += gridDim.x) {
         const bool small = job >= windows;           // the units first, then the small gaskets
         const uint64_t w0 = (small ? job - windows : job) * window;
         const uint32_t begin = (uint32_t)w0;
         const uint32_t end = (uint32_t)min(w0 + window, (uint64_t)total);
         // 32 gaskets at a time from the one that holds the window's first item
-        for (uint32_t i0 = batch_instance(bv.prefix, bv.count, begin);; i0 += 32u) {
+        for (uint32_t i0 = batch_instance_warp(bv.prefix, bv.count, begin, lane);; i0 += 32u) {
             const uint32_t i = i0 + lane;
             const bool have = i < bv.count;
             const uint32_t first = have ? __ldg(bv.prefix + i) : ~0u;
             const uint32_t next = have ? __ldg(bv.prefix + i + 1) : ~0u;
             const int lv = have ? __ldg(bv.level + i) : 0;
+            const uint64_t ba = have ? __ldg(bv.buf_a + i) : 0u, bb = have ? __ldg(bv.buf_b + i) : 0u;
+            const uint64_t src_of = parity ? bb : ba, dst_of = parity ? ba : bb;
             const int r = lv & 0xFF, kk = (lv >> 8) ? (lv >> 8) : k;
             const bool in_window = have && first < end;
             // units of the large gaskets
@@ -280,9 +298,8 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
                 big &= big - 1u;
                 const int rg = __shfl_sync(~0u, r, src), kg = __shfl_sync(~0u, kk, src);
                 const uint32_t fg = __shfl_sync(~0u, first, src), ng = __shfl_sync(~0u, next, src);
-                const uint64_t pa = __ldg(bv.buf_a + i0 + src), pb = __ldg(bv.buf_b + i0 + src);
-                const uint8_t *in = reinterpret_cast<const uint8_t *>(parity ? pb : pa);
-                uint8_t *out = reinterpret_cast<uint8_t *>(parity ? pa : pb);
+                const uint8_t *in = reinterpret_cast<const uint8_t *>(__shfl_sync(~0u, src_of, src));
+                uint8_t *out = reinterpret_cast<uint8_t *>(__shfl_sync(~0u, dst_of, src));
                 const int rbu = rg - 6 - l;
                 ll.set_level((int)lane, rbu);
                 const uint32_t W = pi_word(order, rbu);
@@ -323,9 +340,8 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
                 const int rg = __shfl_sync(~0u, r, gs), kg = __shfl_sync(~0u, kk, gs);
                 const uint32_t tile = lane - __shfl_sync(~0u, excl, gs);
                 WordLane w;
-                const uint64_t pa = __ldg(bv.buf_a + i0 + gs), pb = __ldg(bv.buf_b + i0 + gs);
-                w.in = reinterpret_cast<const uint8_t *>(parity ? pb : pa);
-                w.out = reinterpret_cast<uint8_t *>(parity ? pa : pb);
+                w.in = reinterpret_cast<const uint8_t *>(__shfl_sync(~0u, src_of, gs));
+                w.out = reinterpret_cast<uint8_t *>(__shfl_sync(~0u, dst_of, gs));
                 w.r = rg;
                 w.blocks = w.own = 0u;
                 w.x = w.y = w.ox = w.oy = 0u;
@@ -353,12 +369,13 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
 cudaError_t launch_batch_k(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
                            const LaunchCfg &cfg)
 {
-    if (k == 1) return launch_batch(p, parity, st, cfg);
     if (k < 1 || k > SG_FUSE_MAX) return cudaErrorInvalidValue;
     const int s = p->rho == 16 ? 4 : p->rho == 32 ? 5 : 6;
+    const uint64_t cells = (uint64_t)p->total_tiles * (uint64_t)pow3i(s);
+    // one step: on words from a level-14 gasket's cells on, as for one gasket
+    if (k == 1 && cells < (uint64_t)pow3i(14)) return launch_batch(p, parity, st, cfg);
     // Few tiles: a warp per 16- or 32-tile is the shorter chain, by the same
     // lines as for one gasket (launch_ca_fused in sg_fused.cu, in cells)
-    const uint64_t cells = (uint64_t)p->total_tiles * (uint64_t)pow3i(s);
     if (s == 4 && (cells <= (uint64_t)pow3i(10) || (cells <= (uint64_t)pow3i(11) && k <= 8))) {
         if (k <= 4) return launch_batch_fused_t<4, 4>(p, parity, k, st, cfg);
         if (k <= 8) return launch_batch_fused_t<4, 8>(p, parity, k, st, cfg);
@@ -371,13 +388,16 @@ cudaError_t launch_batch_k(const sg_batch_plan *p, int parity, int k, cudaStream
     static std::atomic<int> occ{0};
     const int l = cells >= (uint64_t)pow3i(13) ? 3 : 2;
     const uint32_t window = (uint32_t)pow3i(l + 6 - s);
+    const bool any_small = p->reserved[1] == 0;
     unsigned grid = 1;
     cudaError_t e = persistent_grid(ca_batch_words_kernel, kWordThreads, 0,
-                                    2u * (((uint64_t)p->total_tiles + window - 1) / window), cfg,
-                                    &grid, &occ);
+                                    (any_small ? 2u : 1u) *
+                                        (((uint64_t)p->total_tiles + window - 1) / window),
+                                    cfg, &grid, &occ);
     if (e != cudaSuccess) return e;
     ca_batch_words_kernel<<<grid, kWordThreads, 0, st>>>(view_of(p), p->total_tiles, parity,
-                                                         cfg.order, k, s, l, window);
+                                                         cfg.order, k, s, l, window,
+                                                         any_small);
     return cudaGetLastError();
 }
 
@@ -425,7 +445,7 @@ sg_status sg_batch_ca_plan_host(int count, const int *levels, const int *steps,
     while ((1 << s) < rho) ++s;
     // validate everything before the image is touched
     uint64_t total = 0;
-    int max_level = 0, max_steps = 0;
+    int max_level = 0, max_steps = 0, min_level = 16;
     for (int i = 0; i < count; ++i) {
         const int r = levels[i];
         if (r < s || r > 16) return SG_EINVAL;        // every gasket holds whole tiles
@@ -434,6 +454,7 @@ sg_status sg_batch_ca_plan_host(int count, const int *levels, const int *steps,
         if (((uintptr_t)buf_a[i] & 15) || ((uintptr_t)buf_b[i] & 15)) return SG_EINVAL;
         total += (uint64_t)pow3i(r - s);
         max_level = std::max(max_level, r);
+        min_level = std::min(min_level, r);
         if (steps != nullptr) max_steps = std::max(max_steps, steps[i]);
         if (total >= (1ull << 32)) return SG_EINVAL;
     }
@@ -460,6 +481,7 @@ sg_status sg_batch_ca_plan_host(int count, const int *levels, const int *steps,
     plan->total_tiles = (uint32_t)total;
     plan->max_level = (uint32_t)max_level;
     plan->reserved[0] = max_steps;                    // launches need k >= every gasket's steps
+    plan->reserved[1] = min_level > kSmallLevel;      // no gasket below level 9 (0: there may be)
     return SG_OK;
 }
 
@@ -490,7 +512,7 @@ sg_status sg_batch_ca_step(const sg_batch_plan *plan, int parity, const sg_launc
     if (!plan_ok(plan) || (parity != 0 && parity != 1) || plan->reserved[0] > 1) return SG_EINVAL;
     LaunchCfg cfg;
     if (!read_launch_opts(opts, &cfg)) return SG_EINVAL;
-    const cudaError_t e = launch_batch(plan, parity, (cudaStream_t)stream, cfg);
+    const cudaError_t e = launch_batch_k(plan, parity, 1, (cudaStream_t)stream, cfg);
     return e == cudaSuccess ? SG_OK : cuda_fail(e);
 }
 

@@ -375,6 +375,10 @@ cudaError_t launch_ca(int r, int s, int map, const uint8_t *in, uint8_t *out,
         SG_S_SWITCH(s, CALL)
 #undef CALL
     }
+    // Large gaskets step on words of 32 tiles whatever the tile side (us on
+    // 64-tiles against words: level 13, 5.8 and 6.8; level 14, 13.4 and 10.3;
+    // level 15, 39.2 and 38.0)
+    if (r >= 14 && cfg.store != kStoreTma) return launch_ca_words(r, in, out, 1, st, cfg);
 #define CALL(S) launch_ca_t<S, kMapLambda>(r, in, out, st, cfg)
     SG_S_SWITCH(s, CALL)
 #undef CALL
