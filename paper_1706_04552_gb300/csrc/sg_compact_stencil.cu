@@ -381,6 +381,258 @@ compact_diffuse_kernel(const float *__restrict__ in, float *__restrict__ out, in
     }
 }
 
+// ---------------------------------------------------------------------------
+// Diffusion, rho >= 16: triples.  The gasket cells come in threes A = (X, Y),
+// B = (X+1, Y), C = (X, Y+1) with X, Y even and (X & Y) == 0.  Of a triple's
+// 4-neighbours, A has B, C and one cell outside at most (the B to its left or
+// the C above it, never both), B has A and the A to its right, C has A and the
+// A below it.  A unit's 729 elements are 243 triples, one per thread in
+// row-major order, so that A and B are consecutive elements, C follows in the
+// next row, and consecutive threads read and write consecutive elements
+// straight from and to HBM; the three outside values go through shared memory
+// (three stores and three loads per triple).  At a tile's corners they come
+// from the neighbouring tile, whose launch index follows from the digits of
+// this one (corner_tile); a warp of its own looks them up ahead.
+//
+// Bound: HBM (reads and writes 8 bytes a cell, contiguous: 17 us at level 15).
+// Each thread keeps two units' loads in flight while it updates two; one
+// barrier per pair (two publishing buffers).  Level 15, rho 64: 36.2 us with
+// five gathers and a table entry per cell, 20.6 here (one unit at a time 23.6;
+// 7 CTAs an SM with 32 registers and spills 30.6, 5 with 40 registers here);
+// rho 16: 44.7 and 23.4; level 10: 6.9 and 2.2.
+// ---------------------------------------------------------------------------
+
+// The tile that touches corner `kind` (0: A, 1: B, 2: C) of tile q in the
+// 4-neighbour graph, as a launch index of the interleaved order (~0u: none).
+// The digits of q are the levels' choices, finest first: 0 the lower, 1 the
+// upper left, 2 the right third.  The finest digits that agree with the corner
+// are skipped; the first that does not says which sibling lies across, and
+// that tile's finer digits are those of the corner it touches with.  *above:
+// at corner A, the tile lies above (else to the left).
+__device__ __forceinline__ uint32_t corner_tile(uint32_t q, uint32_t kind, int rb, bool *above)
+{
+    const uint32_t at = kind == 0u ? 1u : kind == 1u ? 2u : 0u;         // digit at the corner
+    uint32_t pw = 1u, rest = q, d = at;
+    int j = 0;
+    for (; j < rb; ++j, pw *= 3u) {
+        const uint32_t n = rest / 3u;
+        d = rest - 3u * n;
+        rest = n;
+        if (d != at) break;
+    }
+    *above = d == 0u;
+    if (j == rb || (kind != 0u && d != 1u)) return ~0u;    // the gasket's own corner; a diagonal
+    const uint32_t ones = (pw - 1u) / 2u;                  // finer digits all 1
+    return kind == 0u ? q - ones - d * pw + pw + (d == 2u ? 2u * ones : 0u)
+                      : q - at * ones - pw + at * pw + ones;
+}
+
+// Launch index between the walking orders: the digits as levels (interleaved)
+// and dealt to omega_y and omega_x (row-major).
+__device__ __forceinline__ uint32_t rowmajor_to_levels(uint32_t q, int rb)
+{
+    const uint32_t W = (uint32_t)pow3i(rb / 2);
+    uint32_t y = q / W, x = q - y * W, out = 0u, pw = 1u;
+    for (int mu = 1; mu <= rb; ++mu, pw *= 3u) {
+        uint32_t &w = (mu & 1) ? y : x;
+        out += w % 3u * pw;
+        w /= 3u;
+    }
+    return out;
+}
+__device__ __forceinline__ uint32_t levels_to_rowmajor(uint32_t q, int rb)
+{
+    uint32_t y = 0u, x = 0u, py = 1u, px = 1u;
+    for (int mu = 1; mu <= rb; ++mu, q /= 3u) {
+        if (mu & 1) { y += q % 3u * py; py *= 3u; }
+        else { x += q % 3u * px; px *= 3u; }
+    }
+    return y * (uint32_t)pow3i(rb / 2) + x;
+}
+
+// Per triple of a level-S tile, in row-major order: the element of A (B is the
+// next) and of C, and the words the outside values come from (plane * 243 +
+// triple; kNoTriple: none in the tile).  corner: 1, 2, 3 for the tile's corner
+// A, B, C.  (kNoTriple is also the word that holds 0.)
+constexpr uint16_t kNoTriple = 3 * 243;
+template <int S> struct TriplePattern {
+    static constexpr int T = pow3i(S - 1);
+    uint16_t a[T], c[T], rp[T], rq[T], rr[T];
+    uint8_t corner[T];
+};
+template <int S> constexpr TriplePattern<S> make_triple_pattern()
+{
+    constexpr int H = 1 << (S - 1);
+    TriplePattern<S> p{};
+    uint16_t id[H][H] = {};
+    int t = 0;
+    for (int y = 0; y < H; ++y)
+        for (int x = 0; x < H; ++x)
+            if ((x & y) == 0) id[y][x] = (uint16_t)t++;
+    t = 0;
+    for (int y = 0; y < H; ++y) {
+        int m = 0;
+        for (int x = 0; x < H; ++x) m += (x & y) == 0;
+        const int first = t;
+        for (int x = 0; x < H; ++x) {
+            if ((x & y) != 0) continue;
+            p.a[t] = (uint16_t)(3 * first + 2 * (t - first));
+            p.c[t] = (uint16_t)(3 * first + 2 * m + (t - first));
+            p.rp[t] = p.rq[t] = p.rr[t] = kNoTriple;
+            if (x > 0 && ((x - 1) & y) == 0) p.rp[t] = (uint16_t)(243 + id[y][x - 1]);
+            else if (y > 0 && (x & (y - 1)) == 0) p.rp[t] = (uint16_t)(486 + id[y - 1][x]);
+            if (x + 1 < H && ((x + 1) & y) == 0) p.rq[t] = id[y][x + 1];
+            if (y + 1 < H && (x & (y + 1)) == 0) p.rr[t] = id[y + 1][x];
+            if (x == 0 && y == 0) p.corner[t] = 1;
+            if (x == H - 1 && y == 0) p.corner[t] = 2;
+            if (x == 0 && y == H - 1) p.corner[t] = 3;
+            ++t;
+        }
+    }
+    return p;
+}
+__device__ const TriplePattern<4> kTriples4 = make_triple_pattern<4>();
+__device__ const TriplePattern<5> kTriples5 = make_triple_pattern<5>();
+__device__ const TriplePattern<6> kTriples6 = make_triple_pattern<6>();
+template <int S> __device__ __forceinline__ const TriplePattern<S> &triple_pattern()
+{
+    if constexpr (S == 4) return kTriples4;
+    else if constexpr (S == 5) return kTriples5;
+    else return kTriples6;
+}
+
+constexpr int kTripleThreads = 288;      // eight warps of triples, one for the tiles' corners
+constexpr int kTripleUnits = 2;          // units a CTA has in hand at a time
+
+template <int S>
+__global__ void __launch_bounds__(kTripleThreads, 5)
+compact_diffuse_triples_kernel(const float *__restrict__ in, float *__restrict__ out, int r,
+                               int order, uint32_t total, float alpha)
+{
+    constexpr int T = pow3i(S - 1), C = pow3i(S), G = kUnit / C, RHO = 1 << S, N = kTripleUnits;
+    constexpr int EXT = kNoTriple + 1, FLAG = EXT + 3 * G;       // corner values, and what they are
+    __shared__ float pub[2][N][FLAG + 3 * G];
+    const int tid = threadIdx.x;
+    const int rb = r - S;
+    const uint32_t ntiles = total / C, units = (ntiles + G - 1) / G;
+    if (tid < 2 * N) pub[tid & 1][tid >> 1][kNoTriple] = 0.f;
+
+    if (tid >= 256) {
+        // The corner warp: lane i fetches the value outside corner i % 3 of
+        // tile i / 3 of the unit (flag: 0 none, 1 there, 2 there and above).
+        const int lane = tid - 256;
+        const uint32_t g = (uint32_t)lane / 3u, kind = (uint32_t)lane - 3u * g;
+        float e[N], f[N];
+        auto fetch = [&](uint32_t u, int i) {
+            const uint32_t q = u * G + g;
+            e[i] = f[i] = 0.f;
+            if (lane >= 3 * G || q >= ntiles) return;
+            bool above = false;
+            uint32_t nq = corner_tile(order == kOrderInterleaved ? q : rowmajor_to_levels(q, rb),
+                                      kind, rb, &above);
+            if (nq == ~0u) return;
+            if (order != kOrderInterleaved) nq = levels_to_rowmajor(nq, rb);
+            // outside corner A lies the tile's corner B or C, else its corner A
+            const uint32_t at = kind != 0u ? 0u : above ? (uint32_t)C - 1u : (uint32_t)RHO - 1u;
+            e[i] = __ldg(in + (uint64_t)nq * C + at);
+            f[i] = kind == 0u && above ? 2.f : 1.f;
+        };
+        uint32_t u = blockIdx.x;
+#pragma unroll
+        for (int i = 0; i < N; ++i) fetch(min(u + i * gridDim.x, units), i);
+        for (int buf = 0; u < units; buf ^= 1) {
+            if (lane < 3 * G) {
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    pub[buf][i][EXT + lane] = e[i];
+                    pub[buf][i][FLAG + lane] = f[i];
+                }
+            }
+            u += N * gridDim.x;
+#pragma unroll
+            for (int i = 0; i < N; ++i) fetch(min(u + i * gridDim.x, units), i);
+            __syncthreads();
+        }
+        return;
+    }
+
+    const int g = tid / T, t = tid - g * T;
+    const bool mine = tid < 243;
+    uint32_t ea = 0, ec = 0, rp = kNoTriple, rq = kNoTriple, rr = kNoTriple, corner = 0;
+    float da = 2.f, db = 1.f, dc = 1.f;
+    bool left = false;
+    if (mine) {
+        const TriplePattern<S> &pat = triple_pattern<S>();
+        ea = g * C + pat.a[t];
+        ec = g * C + pat.c[t];
+        corner = pat.corner[t];
+        rp = pat.rp[t];
+        rq = pat.rq[t];
+        rr = pat.rr[t];
+        left = rp < 486u;
+        if (rp != kNoTriple) { rp += g * T; da = 3.f; }
+        if (rq != kNoTriple) { rq += g * T; db = 2.f; }
+        if (rr != kNoTriple) { rr += g * T; dc = 2.f; }
+        if (corner == 1u) rp = EXT + 3 * g;
+        if (corner == 2u) rq = EXT + 3 * g + 1;
+        if (corner == 3u) rr = EXT + 3 * g + 2;
+    }
+    float a[N], b[N], c[N];
+    uint32_t u = blockIdx.x;
+    const uint32_t step = gridDim.x * kUnit, to_c = ec - ea;
+    const float *src = in + u * kUnit + ea;
+    float *dst = out + u * kUnit + ea;
+    // the units this thread has a triple in: u < lim (whole ones, or the only one)
+    const uint32_t lim = !mine ? 0u : (uint32_t)g < ntiles ? (ntiles - (uint32_t)g + G - 1) / G : 0u;
+    auto load = [&] {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (u + i * gridDim.x < lim) {
+                a[i] = __ldg(src + i * step);
+                b[i] = __ldg(src + i * step + 1);
+                c[i] = __ldg(src + i * step + to_c);
+            }
+    };
+    load();
+    for (int buf = 0; u < units; buf ^= 1) {
+        float ca[N], cb[N], cc[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float *w = pub[buf][i];
+            ca[i] = a[i];
+            cb[i] = b[i];
+            cc[i] = c[i];
+            if (mine) {
+                w[tid] = a[i];
+                w[243 + tid] = b[i];
+                w[486 + tid] = c[i];
+            }
+        }
+        const uint32_t cur = u;
+        u += N * gridDim.x;
+        src += N * step;
+        load();                             // in flight across the barrier and the update
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if (cur + i * gridDim.x >= lim) break;
+            const float *w = pub[buf][i];
+            const float p = w[rp], q = w[rq], s = w[rr];
+            if (corner != 0u) {
+                const float f = w[FLAG + 3 * g + (int)corner - 1];
+                const float n = f != 0.f ? 1.f : 0.f;
+                if (corner == 1u) { da = 2.f + n; left = f < 2.f; }
+                if (corner == 2u) db = 1.f + n;
+                if (corner == 3u) dc = 1.f + n;
+            }
+            dst[i * step] = diffuse_update(ca[i], left ? p : 0.f, cb[i], left ? 0.f : p, cc[i], da, alpha);
+            dst[i * step + 1] = diffuse_update(cb[i], ca[i], q, 0.f, 0.f, db, alpha);
+            dst[i * step + to_c] = diffuse_update(cc[i], 0.f, 0.f, ca[i], s, dc, alpha);
+        }
+        dst += N * step;
+    }
+}
+
 template <int S>
 cudaError_t launch_ca_t(int r, int order, const uint8_t *in, uint8_t *out, cudaStream_t st,
                         const LaunchCfg &cfg)
@@ -415,16 +667,23 @@ cudaError_t launch_diffuse_t(int r, int order, const float *in, float *out, floa
                              cudaStream_t st, const LaunchCfg &cfg)
 {
     static std::atomic<int> occ{0};
-    static std::atomic<uint64_t> attr{0};
     const uint32_t total = (uint32_t)pow3i(r);
     const uint64_t units = (total + kUnit - 1) / kUnit;
     unsigned grid = 1;
-    auto k = compact_diffuse_kernel<S>;
-    constexpr int smem = StencilSmem<float, S, kDiffHalo, kUnit * 16>::BYTES;
-    cudaError_t e = dyn_smem_grid(k, smem, (units + kUnitWarps - 1) / kUnitWarps, cfg, &grid,
-                                  &occ, &attr);
-    if (e != cudaSuccess) return e;
-    k<<<grid, kUnitThreads, smem, st>>>(in, out, r, order, total, alpha);
+    if constexpr (S >= 4) {
+        auto k = compact_diffuse_triples_kernel<S>;
+        cudaError_t e = persistent_grid(k, kTripleThreads, 0, units, cfg, &grid, &occ);
+        if (e != cudaSuccess) return e;
+        k<<<grid, kTripleThreads, 0, st>>>(in, out, r, order, total, alpha);
+    } else {
+        static std::atomic<uint64_t> attr{0};
+        auto k = compact_diffuse_kernel<S>;
+        constexpr int smem = StencilSmem<float, S, kDiffHalo, kUnit * 16>::BYTES;
+        cudaError_t e = dyn_smem_grid(k, smem, (units + kUnitWarps - 1) / kUnitWarps, cfg, &grid,
+                                      &occ, &attr);
+        if (e != cudaSuccess) return e;
+        k<<<grid, kUnitThreads, smem, st>>>(in, out, r, order, total, alpha);
+    }
     return cudaGetLastError();
 }
 
