@@ -111,6 +111,28 @@ struct LambdaLane {
     }
 };
 
+// The same lambda(omega) by one lane alone, digit by digit: for kernels whose
+// lanes each take a tile of their own (rb steps for 32 tiles, where the warp
+// decode takes one reduction per tile).  W = pi_word(order, rb).
+__device__ __forceinline__ uint2 lambda_block(uint32_t q, int rb, int order, uint32_t W)
+{
+    uint32_t lx = 0, ly = 0;
+    uint32_t w = q, v = 0;                 // the word the next digit comes from, the other
+    if (order == kOrderRowMajor) {
+        w = q / W;                         // omega_y first (Eq. beta, odd mu)
+        v = q - w * W;
+    }
+    for (int j = 0; j < rb; ++j) {
+        const uint32_t n = w / 3u, beta = w - 3u * n;
+        const uint32_t dx = beta >> 1;
+        lx |= dx << j;
+        ly |= (beta - dx) << j;
+        w = n;
+        if (order == kOrderRowMajor) { w = v; v = n; }
+    }
+    return make_uint2(lx, (1u << rb) - 1u - ly);
+}
+
 // A persistent loop advances the launch index q by a fixed stride; the two
 // words (a, b) = (q mod W, q div W) are stepped incrementally instead of
 // divided every time.
@@ -200,6 +222,11 @@ template <typename T, int VK> struct CellValue {
     {
         return VK == kValLinear31 ? tx * 31u + ty : (ty << r) | tx;
     }
+    // The hash bits the values are cut from: the uint8 value is the top byte.
+    __device__ __forceinline__ uint32_t hash_word(uint32_t base, uint32_t koff) const
+    {
+        return splitmix64_hi_state(((uint32_t)seedmix ^ base) ^ koff, (uint32_t)(seedmix >> 32));
+    }
     __device__ __forceinline__ T operator()(uint32_t base, uint32_t koff) const
     {
         if constexpr (VK == kValConst) {
@@ -210,8 +237,7 @@ template <typename T, int VK> struct CellValue {
         } else {
             // bits 32..63 of the hash; (seedmix ^ base) is the same for the
             // whole tile, so it is computed once per tile
-            const uint32_t hi = splitmix64_hi_state(((uint32_t)seedmix ^ base) ^ koff,
-                                                    (uint32_t)(seedmix >> 32));
+            const uint32_t hi = hash_word(base, koff);
             if constexpr (sizeof(T) == 1) return (T)(hi >> 24);
             else return (float)(hi >> 8) * (1.0f / 16777216.0f);
         }

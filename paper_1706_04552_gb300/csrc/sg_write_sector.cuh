@@ -28,9 +28,12 @@
 //     sector, reading what it does not hold from DRAM.  Only gasket cells ever
 //     change.
 //
-// The tile of each unit comes from the lambda(omega) decode of Theorem 1
-// (LambdaLane, one warp reduction per tile; the warp decodes the tiles its 32
-// units span, one after the other) or from the bounding-box identity map, in
+// Lanes walk whole units, or one row group each (`pieces`; 32 lanes still work on
+// the same rows of 32 units).
+//
+// The tile of each unit comes from the lambda(omega) decode of Theorem 1, every
+// lane its own (lambda_block: 32 warp reductions one after the other took 3.5
+// of 11.8 us at level 11), or from the bounding-box identity map, in
 // which a lane whose tile holds no gasket cell does nothing, as the empty
 // blocks of the paper's bounding-box launch do.
 #pragma once
@@ -65,6 +68,9 @@ template <typename T, int S> struct SectorShape {
     static constexpr int LU = sizeof(T) == 1 ? 5 : (S < 5 ? S : 5);   // log2(US)
     static constexpr int SUB = S - LU;                            // unit levels in a tile
     static constexpr bool OK = (1 << S) * (int)sizeof(T) >= 32;
+    // row groups of a unit that can be worked on apart: 4 rows of a uint8
+    // unit; 8 rows of one column of sectors of a float32 unit
+    static constexpr uint32_t PIECES = sizeof(T) == 1 ? 8u : (uint32_t)((US / 8) * (US / 8));
 };
 
 // The value of each cell of one row of a unit: a per-row part and a per-cell
@@ -100,9 +106,10 @@ template <typename T, int VK> struct RowValue {
 template <int VK, int MODE>
 __device__ __forceinline__ void sector_unit_u8(uint8_t *__restrict__ grid, int r, uint32_t x0,
                                                uint32_t y0, uint64_t seedmix,
-                                               RowValue<uint8_t, VK> rv)
+                                               RowValue<uint8_t, VK> rv, uint32_t th0,
+                                               uint32_t th1)
 {
-    for (uint32_t th = 0; th < 8u; ++th) {
+    for (uint32_t th = th0; th < th1; ++th) {
         uint32_t old[4][8];
         if constexpr (MODE == kStoreMerge) {
 #pragma unroll
@@ -151,11 +158,12 @@ __device__ __forceinline__ void sector_unit_u8(uint8_t *__restrict__ grid, int r
 template <int VK, int MODE, int US>
 __device__ __forceinline__ void sector_unit_f32(float *__restrict__ grid, int r, uint32_t x0,
                                                 uint32_t y0, uint64_t seedmix,
-                                                RowValue<float, VK> rv)
+                                                RowValue<float, VK> rv, uint32_t p0, uint32_t p1)
 {
     constexpr uint32_t NS = US / 8;                   // sectors per row, row groups
-    for (uint32_t th = 0; th < NS; ++th) {
-        for (uint32_t sx = 0; sx < NS; ++sx) {
+    {
+        for (uint32_t p = p0; p < p1; ++p) {          // th = p / NS, sx = p mod NS
+            const uint32_t th = p / NS, sx = p % NS;
             if ((sx & th) != 0u) continue;            // uniform: no gasket cell
             const uint32_t xs = x0 + 8u * sx;
             uint32_t old[8][8];
@@ -188,7 +196,8 @@ __device__ __forceinline__ void sector_unit_f32(float *__restrict__ grid, int r,
 
 template <typename T, int VK, int S, int MAP, int MODE>
 __global__ void __launch_bounds__(kSectorThreads)
-write_sector_kernel(T *__restrict__ grid, int r, int order, uint64_t vs, uint64_t ntiles)
+write_sector_kernel(T *__restrict__ grid, int r, int order, uint64_t vs, uint64_t ntiles,
+                    uint32_t pieces)
 {
     using SS = SectorShape<T, S>;
     constexpr int SUB = SS::SUB;
@@ -203,32 +212,26 @@ write_sector_kernel(T *__restrict__ grid, int r, int order, uint64_t vs, uint64_
     rv.seed_hi = (uint32_t)(seedmix >> 32);
     rv.cval = (uint32_t)vs;
     rv.row = 0;
-    LambdaLane ll;
-    uint32_t W = 1;
-    if constexpr (MAP != kMapBBox) {
-        ll.init(lane, rb, order);
-        W = pi_word(order, rb);
-    }
+    const uint32_t W = MAP == kMapBBox ? 1u : pi_word(order, rb);
+    const uint64_t groups = (nunits + 31) / 32;              // 32 units side by side
 
-    for (uint64_t task = warp0; task * 32 < nunits; task += nwarps) {
-        const uint64_t unit = task * 32 + (uint64_t)lane;
+    for (uint64_t task = warp0; task < groups * pieces; task += nwarps) {
+        // pieces = 1: the whole units; else the units' piece-th row group
+        const uint64_t gi = pieces == 1u ? task : task / pieces;
+        const uint32_t piece = (uint32_t)(task - gi * pieces);
+        const uint32_t p0 = pieces == 1u ? 0u : piece, p1 = pieces == 1u ? SS::PIECES : piece + 1u;
+        const uint64_t unit = gi * 32 + (uint64_t)lane;
         const uint64_t q = unit / PER;
         const uint32_t u = (uint32_t)(unit - q * PER);
         uint32_t bx = kNoUnit, by = kNoUnit;
-        if constexpr (MAP == kMapBBox) {
-            if (unit < nunits) {
+        if (unit < nunits) {
+            if constexpr (MAP == kMapBBox) {
                 const uint32_t tx = (uint32_t)(q & ((1ull << rb) - 1)), tyy = (uint32_t)(q >> rb);
                 if ((tx & tyy) == 0u) { bx = tx; by = tyy; }
-            }
-        } else {
-            // the warp decodes the tiles its units span, one per reduction
-            const uint64_t q_first = (task * 32) / PER;
-            const uint64_t last = task * 32 + 31 < nunits ? task * 32 + 31 : nunits - 1;
-            const uint64_t q_last = last / PER;
-            for (uint64_t t = q_first; t <= q_last; ++t) {
-                const uint32_t b = (uint32_t)t / W, a = (uint32_t)t - b * W;
-                const uint2 c = ll.decode(a, b);
-                if (t == q && unit < nunits) { bx = c.x; by = c.y; }
+            } else {
+                const uint2 c = lambda_block((uint32_t)q, rb, order, W);
+                bx = c.x;
+                by = c.y;
             }
         }
         // the unit inside its tile: for lambda the level-SUB gasket's units
@@ -238,10 +241,11 @@ write_sector_kernel(T *__restrict__ grid, int r, int order, uint64_t vs, uint64_
         if (bx == kNoUnit || (ux & uy) != 0u) continue;
         const uint32_t x0 = (bx << S) + ux * SS::US, y0 = (by << S) + uy * SS::US;
         if constexpr (sizeof(T) == 1)
-            sector_unit_u8<VK, MODE>(reinterpret_cast<uint8_t *>(grid), r, x0, y0, seedmix, rv);
+            sector_unit_u8<VK, MODE>(reinterpret_cast<uint8_t *>(grid), r, x0, y0, seedmix, rv, p0,
+                                     p1);
         else
             sector_unit_f32<VK, MODE, SS::US>(reinterpret_cast<float *>(grid), r, x0, y0,
-                                              seedmix, rv);
+                                              seedmix, rv, p0, p1);
     }
 }
 
@@ -257,7 +261,17 @@ cudaError_t launch_write_sector(int r, T *grid, uint64_t vs, uint64_t ntiles, cu
         return cudaErrorNotSupported;
     } else {
         constexpr uint64_t PER = M == kMapBBox ? (1ull << (2 * SS::SUB)) : (uint64_t)pow3i(SS::SUB);
-        const uint64_t tasks = (ntiles * PER + 31) / 32;
+        const uint64_t groups = (ntiles * PER + 31) / 32;
+        // A lane that walks a whole unit alone is a chain of 32 rows: row groups
+        // apart are shorter and many more (merge, us, whole and apart: float32,
+        // rho 16, level 11, 8.1 and 3.8; rho 64, level 14, 33.2 and 23.7, level
+        // 16, 351 and 242; uint8, level 11, 16.9 and 5.2, level 15, 35.7 and
+        // 35.3).  Only the uint8 grid of level 16 (5536 groups) keeps whole
+        // units, 114 against 121, and the bounding box, where most of a
+        // group's units are empty.
+        const uint32_t pieces =
+            M != kMapBBox && (sizeof(T) == 4 || groups <= 2048) ? SS::PIECES : 1u;
+        const uint64_t tasks = groups * pieces;
         const uint64_t units = (tasks + kSectorThreads / 32 - 1) / (kSectorThreads / 32);
         unsigned grid_ctas = 1;
         cudaError_t e;
@@ -266,19 +280,22 @@ cudaError_t launch_write_sector(int r, T *grid, uint64_t vs, uint64_t ntiles, cu
             auto kern = write_sector_kernel<T, VK, S, M, kStoreMerge>;
             e = persistent_grid(kern, kSectorThreads, 0, units, cfg, &grid_ctas, &occ);
             if (e != cudaSuccess) return e;
-            kern<<<grid_ctas, kSectorThreads, 0, st>>>(grid, r, cfg.order, vs, ntiles);
+            kern<<<grid_ctas, kSectorThreads, 0, st>>>(grid, r, cfg.order, vs, ntiles,
+                                                       pieces);
         } else if (cfg.store == kStoreMasked) {
             static std::atomic<int> occ{0};
             auto kern = write_sector_kernel<T, VK, S, M, kStoreMasked>;
             e = persistent_grid(kern, kSectorThreads, 0, units, cfg, &grid_ctas, &occ);
             if (e != cudaSuccess) return e;
-            kern<<<grid_ctas, kSectorThreads, 0, st>>>(grid, r, cfg.order, vs, ntiles);
+            kern<<<grid_ctas, kSectorThreads, 0, st>>>(grid, r, cfg.order, vs, ntiles,
+                                                       pieces);
         } else {
             static std::atomic<int> occ{0};
             auto kern = write_sector_kernel<T, VK, S, M, kStoreSector>;
             e = persistent_grid(kern, kSectorThreads, 0, units, cfg, &grid_ctas, &occ);
             if (e != cudaSuccess) return e;
-            kern<<<grid_ctas, kSectorThreads, 0, st>>>(grid, r, cfg.order, vs, ntiles);
+            kern<<<grid_ctas, kSectorThreads, 0, st>>>(grid, r, cfg.order, vs, ntiles,
+                                                       pieces);
         }
         return cudaGetLastError();
     }
