@@ -87,8 +87,7 @@ template <typename T> __host__ __device__ constexpr int write_stage_bytes()
 
 // WIDE: stage each unit in shared memory and store it in whole aligned
 // 16-byte chunks (for a destination in host memory, across the host link);
-// otherwise every lane stores its values directly (device memory, where the
-// staging's extra registers cost more than the wide stores save).
+// otherwise every lane stores its values directly (device memory, rho <= 8).
 template <typename T, int VK, int S, bool WIDE>
 __global__ void __launch_bounds__(kUnitThreads)
 compact_write_kernel(T *__restrict__ compact, int r, int order, uint32_t total, uint64_t vs)
@@ -163,6 +162,104 @@ compact_write_kernel(T *__restrict__ compact, int r, int order, uint32_t total, 
     }
 }
 
+// rho >= 16, device memory: a lane computes four consecutive elements at an
+// aligned address and stores them at once.  729 u mod 4 = u mod 4, and a warp's
+// units are a multiple of 8 apart, so all of them start at the same place
+// within four elements: the value-key offsets of a lane's 24 elements never
+// change and stay in registers, and the loop over units touches no shared
+// memory.  Only a unit's first and last words, shared with its neighbours,
+// store element by element.
+//
+// Bound: integer issue (the hash: ALU 68 %, and moving its adds and shifts to
+// the multipliers was slower, 41.3 and 43.7 us).  uint8, level 16, with a table
+// load and a byte store per element and here: rho 64, 43.5 and 39.0 us; rho 16,
+// 75.2 and 51.5 (a shuffle per element finds its tile's base); float32, level
+// 15, rho 16: 29.2 and 20.1.
+template <typename T, int VK, int S>
+__global__ void __launch_bounds__(kUnitThreads)
+compact_write4_kernel(T *__restrict__ compact, int r, int order, uint32_t total, uint64_t vs)
+{
+    constexpr int C = CompactPattern<S>::C, G = CompactPattern<S>::G, WORDS = 6;
+    static_assert(G <= 32, "a lane per tile of the unit");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rb = r - S;
+    const uint32_t ntiles = total / C, units = (total + kUnit - 1) / kUnit;
+    const CellValue<T, VK> cv{vs * kGoldenGamma, (uint32_t)vs};
+    const uint32_t W = pi_word(order, rb);
+    LambdaLane ll;
+    ll.init(lane, rb, order);
+    const uint32_t u0 = blockIdx.x * kUnitWarps + warp, nwarps = gridDim.x * kUnitWarps;
+    // elements before the unit's first aligned word of four
+    const int lead = (int)(((uint32_t)(reinterpret_cast<uintptr_t>(compact) / sizeof(T)) + u0) & 3u);
+    // word i of the lane: elements 4 (lane + 32 i) - lead + 0..3 of the unit
+    uint32_t koff[WORDS][4], tile[WORDS];
+#pragma unroll
+    for (int i = 0; i < WORDS; ++i) {
+        tile[i] = 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = min(max(4 * (lane + 32 * i) - lead + k, 0), kUnit - 1);
+            const uint32_t cell = unit_cell<S>(c);
+            koff[i][k] = CellValue<T, VK>::offset_of((cell >> 10) & 0x3Fu, cell >> 16, r);
+            tile[i] |= (cell & 0x3FFu) << (8 * k);
+        }
+    }
+    for (uint32_t u = u0; u < units; u += nwarps) {
+        uint32_t vbase = 0u;                           // of tile `lane` of the unit
+        if constexpr (G == 1) {
+            const uint32_t bq = u / W, aq = u - bq * W;
+            const uint2 b = ll.decode(aq, bq);
+            vbase = CellValue<T, VK>::base_of(b.x << S, b.y << S, r);
+        } else {
+            const uint32_t q = u * G + (uint32_t)min(lane, G - 1);
+            if (q < ntiles) {
+                const uint2 b = lambda_block(q, rb, order, W);
+                vbase = CellValue<T, VK>::base_of(b.x << S, b.y << S, r);
+            }
+        }
+        const int cnt = (int)min((uint32_t)kUnit, total - u * kUnit);
+        T *dst = compact + (uint64_t)u * kUnit - lead + 4 * lane;
+#pragma unroll
+        for (int i = 0; i < WORDS; ++i, dst += 128) {
+            uint32_t base[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                base[k] = G == 1 ? vbase
+                                 : __shfl_sync(~0u, vbase, (int)((tile[i] >> (8 * k)) & 31u));
+            const int e = 4 * (lane + 32 * i) - lead;
+            if constexpr (sizeof(T) == 1) {
+                // the four values as one word: the top bytes of the hash words
+                uint32_t v[4], sel = VK == kValHash ? 0x0073u : 0x0040u;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (VK == kValHash) v[k] = cv.hash_word(base[k], koff[i][k]);
+                    else v[k] = cv(base[k], koff[i][k]);
+                }
+                const uint32_t w = __byte_perm(__byte_perm(v[0], v[1], sel),
+                                               __byte_perm(v[2], v[3], sel), 0x5410);
+                if (e >= 0 && e + 3 < cnt) {
+                    *reinterpret_cast<uint32_t *>(dst) = w;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (e + k >= 0 && e + k < cnt) dst[k] = (uint8_t)(w >> (8 * k));
+                }
+            } else {
+                float v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = cv(base[k], koff[i][k]);
+                if (e >= 0 && e + 3 < cnt) {
+                    *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (e + k >= 0 && e + k < cnt) dst[k] = v[k];
+                }
+            }
+        }
+    }
+}
+
 template <typename T, int S, bool WIDE> constexpr int write_smem_bytes()
 {
     return write_stage_offset<S>() + (WIDE ? kUnitWarps * write_stage_bytes<T>() : 0);
@@ -191,17 +288,26 @@ cudaError_t launch_write_t(int r, int order, T *compact, uint64_t vs, cudaStream
                            const LaunchCfg &cfg)
 {
     static std::atomic<int> occ{0};
-    static std::atomic<uint64_t> attr{0};
     const uint32_t total = (uint32_t)pow3i(r);
     const uint64_t units = (total + kUnit - 1) / kUnit;
     unsigned grid = 1;
-    auto k = compact_write_kernel<T, VK, S, WIDE>;
-    constexpr int smem = write_smem_bytes<T, S, WIDE>();
-    cudaError_t e = dyn_smem_grid(k, smem, (units + kUnitWarps - 1) / kUnitWarps, cfg, &grid,
-                                  &occ, &attr);
-    if (e != cudaSuccess) return e;
-    k<<<grid, kUnitThreads, smem, st>>>(compact, r, order, total, vs);
-    return cudaGetLastError();
+    if constexpr (!WIDE && S >= 4) {
+        auto k4 = compact_write4_kernel<T, VK, S>;
+        cudaError_t e = persistent_grid(k4, kUnitThreads, 0, (units + kUnitWarps - 1) / kUnitWarps,
+                                        cfg, &grid, &occ);
+        if (e != cudaSuccess) return e;
+        k4<<<grid, kUnitThreads, 0, st>>>(compact, r, order, total, vs);
+        return cudaGetLastError();
+    } else {
+        static std::atomic<uint64_t> attr{0};
+        auto k = compact_write_kernel<T, VK, S, WIDE>;
+        constexpr int smem = write_smem_bytes<T, S, WIDE>();
+        cudaError_t e = dyn_smem_grid(k, smem, (units + kUnitWarps - 1) / kUnitWarps, cfg, &grid,
+                                      &occ, &attr);
+        if (e != cudaSuccess) return e;
+        k<<<grid, kUnitThreads, smem, st>>>(compact, r, order, total, vs);
+        return cudaGetLastError();
+    }
 }
 
 #define SG_COMPACT_S_SWITCH(s, CALL)         \

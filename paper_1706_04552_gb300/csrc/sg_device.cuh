@@ -173,27 +173,29 @@ enum : int { kValConst = 0, kValLinear31 = 1, kValHash = 2 };
 // arithmetic written on 32-bit halves: the state's high half is the
 // constant high half of seedmix, each 64-bit shift is one funnel shift per
 // half, and the second product needs only its high half.
+//
+// The ALU pipe bounds the hash, the multiplies run beside it, so what can go to
+// the multipliers does: the sum s + gamma is one 64-bit add of a 32-bit value;
+// its high half takes one of two values (carry or not), so the first xor-shift
+// of the high half and its product with M1's low half are two constants per
+// seed, and one multiply-add, linear in the carry, yields the right one.
 __device__ __forceinline__ uint32_t splitmix64_hi_state(uint32_t s_lo, uint32_t s_hi)
 {
-    constexpr uint32_t G_LO = (uint32_t)kGoldenGamma, G_HI = (uint32_t)(kGoldenGamma >> 32);
     constexpr uint64_t M1 = 0xBF58476D1CE4E5B9ull, M2 = 0x94D049BB133111EBull;
     constexpr uint32_t M1_LO = (uint32_t)M1, M1_HI = (uint32_t)(M1 >> 32);
     constexpr uint32_t M2_LO = (uint32_t)M2, M2_HI = (uint32_t)(M2 >> 32);
-    // z = s + gamma: the high half is one of two values (carry or not), and
-    // so is the high half after the first xor-shift; both pairs depend only
-    // on the seed and are computed once per thread
-    const uint32_t zh0 = s_hi + G_HI, zh1 = zh0 + 1u;
-    const uint32_t th0 = zh0 ^ (zh0 >> 30), th1 = zh1 ^ (zh1 >> 30);
-    const uint32_t z_lo = s_lo + G_LO;
-    const bool carry = z_lo < s_lo;
-    const uint32_t z_hi = carry ? zh1 : zh0;
-    // z ^= z >> 30
+    // per seed (loop invariants): t_hi * M1_LO = z_hi * D + E for z_hi = zh0, zh0 + 1
+    const uint32_t zh0 = s_hi + (uint32_t)(kGoldenGamma >> 32), zh1 = zh0 + 1u;
+    const uint32_t A0 = (zh0 ^ (zh0 >> 30)) * M1_LO, A1 = (zh1 ^ (zh1 >> 30)) * M1_LO;
+    const uint32_t D = A1 - A0, E = A0 - zh0 * D;
+    const uint64_t z = (uint64_t)s_lo + (((uint64_t)s_hi << 32) + kGoldenGamma);
+    const uint32_t z_lo = (uint32_t)z, z_hi = (uint32_t)(z >> 32);
+    // z ^= z >> 30, low half
     const uint32_t t_lo = z_lo ^ __funnelshift_r(z_lo, z_hi, 30);
-    const uint32_t t_hi = carry ? th1 : th0;
     // z *= M1 (mod 2^64)
-    const uint64_t p = (uint64_t)t_lo * M1_LO;
+    const uint64_t p = (uint64_t)t_lo * M1_LO + ((uint64_t)E << 32);
     const uint32_t y_lo = (uint32_t)p;
-    const uint32_t y_hi = (uint32_t)(p >> 32) + t_lo * M1_HI + t_hi * M1_LO;
+    const uint32_t y_hi = (uint32_t)(p >> 32) + t_lo * M1_HI + z_hi * D;
     // z ^= z >> 27
     const uint32_t w_lo = y_lo ^ __funnelshift_r(y_lo, y_hi, 27);
     const uint32_t w_hi = y_hi ^ (y_hi >> 27);
