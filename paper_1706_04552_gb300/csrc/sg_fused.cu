@@ -19,10 +19,11 @@
 // The CA runs bit-sliced: one warp per tile on rows of bits (32 cells per word
 // operation), and under lambda on large gaskets one bit per tile, 32 tiles per
 // word operation (sg_words.cuh).
-// Diffusion at tile sides 32 and 64 runs one warp per 32 x 32 unit with the
-// 9-cell gasket blocks of 4 x 4 cells held in registers (diffuse_warp_fused_
-// kernel, below); at side 16 one CTA per tile on float4 chunks
-// (diffuse_fused_kernel).  Either way each cell's result is the single step's,
+// Diffusion under lambda runs up to 8 steps on one warp per 64-tile
+// (sg_diffuse_tile.cu).  Here are the bounding-box map and 9 to 16 steps: at tile
+// sides 32 and 64 one warp per 32 x 32 unit with the 9-cell gasket blocks of
+// 4 x 4 cells held in registers (diffuse_warp_fused_kernel, below); at side 16
+// one CTA per tile on float4 chunks (diffuse_fused_kernel).  Either way each cell's result is the single step's,
 // so k fused steps equal k single steps.  HBM moves about the tile bytes once
 // in and once out per launch instead of per step.
 //
@@ -681,9 +682,18 @@ cudaError_t launch_diffuse_fused(int r, int s, int map, const float *in, float *
         SG_FUSED_SWITCH(s, k, CALL);
 #undef CALL
     }
+    // up to 8 steps: a warp per 64-tile (sg_diffuse_tile.cu), except where a CTA
+    // per 16-tile is the shorter chain (us, 2 and 4 steps: level 8, 2.6 and 3.0
+    // against 3.1 and 3.2; level 10, 3.8 and 4.8 against 3.0 and 3.2)
+    if (k <= 8 && r >= 6 && !(s == 4 && r <= 9 && k <= 4))
+        return launch_diffuse_tile(r, in, out, alpha, k, st, cfg);
+    if (s == 6) return launch_diffuse_fused_t<6, 16, kMapLambda>(r, in, out, alpha, k, st, cfg);
 #define CALL(S, KH) launch_diffuse_fused_t<S, KH, kMapLambda>(r, in, out, alpha, k, st, cfg)
-    SG_FUSED_SWITCH(s, k, CALL);
+    const int kh = k <= 4 ? 4 : k <= 8 ? 8 : 16;
+    if (s == 4) return kh == 4 ? CALL(4, 4) : kh == 8 ? CALL(4, 8) : CALL(4, 16);
+    if (s == 5) return kh == 4 ? CALL(5, 4) : kh == 8 ? CALL(5, 8) : CALL(5, 16);
 #undef CALL
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace sg

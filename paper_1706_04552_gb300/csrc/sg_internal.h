@@ -55,6 +55,9 @@ cudaError_t launch_ca_fused(int r, int s, int map, const uint8_t *in, uint8_t *o
 // k (1 .. 16) CA steps under lambda on words of 32 64-tiles (level >= 4).
 cudaError_t launch_ca_words(int r, const uint8_t *in, uint8_t *out, int k, cudaStream_t st,
                             const LaunchCfg &cfg);
+// k (1 .. 8) diffusion steps under lambda, one warp per 64-tile (level >= 6).
+cudaError_t launch_diffuse_tile(int r, const float *in, float *out, float alpha, int k,
+                                cudaStream_t st, const LaunchCfg &cfg);
 cudaError_t launch_diffuse_fused(int r, int s, int map, const float *in, float *out,
                                  float alpha, int k, cudaStream_t st, const LaunchCfg &cfg);
 cudaError_t launch_block_map(int rb, int order, uint32_t *bx, uint32_t *by,

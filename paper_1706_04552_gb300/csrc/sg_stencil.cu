@@ -1,6 +1,10 @@
 // sg_stencil.cu -- per-cell stencils over the embedded gasket: the B3/S23
 // cellular automaton (uint8) and explicit diffusion (float32).
 //
+// Under lambda, diffusion from level 6 on runs in sg_diffuse_tile.cu and the CA
+// from level 14 on in sg_words.cuh; the kernels here serve the bounding box, the
+// smaller gaskets and tensor-copy staging.
+//
 // The embedded layout keeps (x +- 1, y +- 1) a neighbourhood of the gasket
 // (Section I), so a tile's update needs the tile plus a one-cell halo.  The
 // CA at rho = 32, 64 and diffusion at rho = 16, 32 run one warp per tile
@@ -329,7 +333,9 @@ cudaError_t launch_diffuse_t(int r, const float *in, float *out, float alpha,
             return launch_diffuse_tma<S, MAP>(r, in, out, alpha, ntiles, st, cfg);
         else return cudaErrorNotSupported;
     }
-    if constexpr (S == 4 || S == 5) {
+    if constexpr (S == 6 && MAP == kMapLambda) {
+        return cudaErrorInvalidValue;      // 64-tiles under lambda: sg_diffuse_tile.cu
+    } else if constexpr (S == 4 || S == 5) {
         static std::atomic<int> occ{0};
         static std::atomic<uint64_t> attr{0};
         auto k = diffuse_warp_kernel<S, MAP>;
@@ -392,6 +398,12 @@ cudaError_t launch_diffuse(int r, int s, int map, const float *in, float *out,
         SG_S_SWITCH(s, CALL)
 #undef CALL
     }
+    // A warp per 64-tile with every cell in a register, whatever the tile side;
+    // 16-tiles on small gaskets are the one shorter chain (us, 16-tiles against
+    // it: level 8, 2.6 and 2.9; level 10, 2.8 and 3.1; level 11, 3.2 and 3.0;
+    // level 14, 33.3 and 26.4)
+    if (r >= 6 && cfg.store != kStoreTma && !(s == 4 && r <= 10))
+        return launch_diffuse_tile(r, in, out, alpha, 1, st, cfg);
 #define CALL(S) launch_diffuse_t<S, kMapLambda>(r, in, out, alpha, st, cfg)
     SG_S_SWITCH(s, CALL)
 #undef CALL
