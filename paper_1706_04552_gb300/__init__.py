@@ -112,6 +112,8 @@ class SchedResult(ctypes.Structure):
 def lib() -> ctypes.CDLL:
     """Load libsg.so (built in-tree by ``paper_1706_04552_gb300.build``)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -321,14 +323,32 @@ def sg_launch_stats(r, rho, map_kind):
 
 # ------------------------------------------------------------- tensor layer
 
+# torch, and its two calls that every launch makes (the current stream's handle
+# and the current device, as integers); bound on the first tensor call.  A
+# call's own cost, 9 to 10 us a launch, was mostly these through their public
+# wrappers and repeated imports; it is about half now.
+torch = _raw_stream = _current_device = None
+
+
+def _bind_torch():
+    global torch, _raw_stream, _current_device
+    if torch is None:
+        import torch as t
+        raw = getattr(t._C, "_cuda_getCurrentRawStream", None)
+        dev = getattr(t._C, "_cuda_getDevice", None)
+        _raw_stream = raw or (lambda i: t.cuda.current_stream(i).cuda_stream)
+        _current_device = dev or t.cuda.current_device
+        torch = t
+    return torch
+
+
 def _map_id(m) -> int:
     return MAPS[m] if isinstance(m, str) else int(m)
 
 
 def _stream_handle(t, stream):
-    import torch
     if stream is None:
-        return torch.cuda.current_stream(t.device).cuda_stream
+        return _raw_stream(t.get_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -340,16 +360,18 @@ class _NoDeviceSwitch:
         return False
 
 
+_NO_SWITCH = _NoDeviceSwitch()
+
+
 def _on_device(t):
     """Make t's device current for the call (skipped when it already is)."""
-    import torch
-    if t.device.index is None or t.device.index == torch.cuda.current_device():
-        return _NoDeviceSwitch()
+    _bind_torch()
+    if t.get_device() == _current_device():
+        return _NO_SWITCH
     return torch.cuda.device(t.device)
 
 
 def _grid_check(t, r, dtypes, name):
-    import torch
     n = 1 << r
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: expected a CUDA tensor (there is no CPU path)")
@@ -362,7 +384,7 @@ def _grid_check(t, r, dtypes, name):
 def map_write(grid, r: int, rho: int, map="lambda", value="hash", value_or_seed=1,
               stream=None, order=None, store=None, ctas_per_sm=None):
     """Map-and-write pass on a CUDA tensor (uint8 or float32, n*n elements)."""
-    import torch
+    _bind_torch()
     _grid_check(grid, r, (torch.uint8, torch.float32), "grid")
     dt = DTYPES["u8"] if grid.dtype == torch.uint8 else DTYPES["f32"]
     vk = VALUES[value] if isinstance(value, str) else int(value)
@@ -381,7 +403,7 @@ def map_write_host(host_grid, dev_grid, r: int, rho: int, map="lambda", value="h
     launches the pass, and copies the result back, all on one stream.
     Returns without synchronising; the copy back is complete once the stream
     is."""
-    import torch
+    _bind_torch()
     if host_grid.is_cuda or not host_grid.is_contiguous():
         raise TypeError("host_grid: expected a contiguous CPU tensor")
     if host_grid.dtype != dev_grid.dtype or host_grid.numel() != dev_grid.numel():
@@ -400,7 +422,7 @@ def map_write_mapped(host_grid, r: int, rho: int, map="lambda", value="hash", va
     place by the kernel over the host link (sg_map_write_mapped).  Returns
     without synchronising: the result is in ``host_grid`` once the stream is
     complete."""
-    import torch
+    _bind_torch()
     if host_grid.is_cuda or not host_grid.is_contiguous() or not host_grid.is_pinned():
         raise TypeError("host_grid: expected a contiguous pinned CPU tensor")
     if host_grid.dtype not in (torch.uint8, torch.float32):
@@ -426,7 +448,7 @@ def ca_step(inp, out, r: int, rho: int, map="lambda", stream=None, order=None,
             ctas_per_sm=None, staging=None):
     """One CA step; staging="tma" stages each tile and its halo with one
     bulk tensor copy (rho 32 and 64) instead of 16-byte chunk copies."""
-    import torch
+    _bind_torch()
     _grid_check(inp, r, (torch.uint8,), "in")
     _grid_check(out, r, (torch.uint8,), "out")
     opts = launch_opts(order, _staging_store(staging), ctas_per_sm)
@@ -440,7 +462,7 @@ def diffuse_step(inp, out, r: int, rho: int, alpha: float = 0.2, map="lambda",
                  stream=None, order=None, ctas_per_sm=None, staging=None):
     """One diffusion step; staging="tma" stages each tile and its halo with
     one bulk tensor copy (rho 16 and 32) instead of 16-byte chunk copies."""
-    import torch
+    _bind_torch()
     _grid_check(inp, r, (torch.float32,), "in")
     _grid_check(out, r, (torch.float32,), "out")
     opts = launch_opts(order, _staging_store(staging), ctas_per_sm)
@@ -465,7 +487,7 @@ FUSE_MAX = 16     # SG_FUSE_MAX: most steps one sg_ca_steps / sg_diffuse_steps l
 def ca_steps(inp, out, r: int, rho: int, k: int, map="lambda", stream=None, order=None,
              ctas_per_sm=None):
     """k CA steps in one launch: out = step^k(inp); inp is left unchanged."""
-    import torch
+    _bind_torch()
     _grid_check(inp, r, (torch.uint8,), "in")
     _grid_check(out, r, (torch.uint8,), "out")
     opts = launch_opts(order, None, ctas_per_sm)
@@ -478,7 +500,7 @@ def ca_steps(inp, out, r: int, rho: int, k: int, map="lambda", stream=None, orde
 def diffuse_steps(inp, out, r: int, rho: int, k: int, alpha: float = 0.2, map="lambda",
                   stream=None, order=None, ctas_per_sm=None):
     """k diffusion steps in one launch: out = step^k(inp); inp is left unchanged."""
-    import torch
+    _bind_torch()
     _grid_check(inp, r, (torch.float32,), "in")
     _grid_check(out, r, (torch.float32,), "out")
     opts = launch_opts(order, None, ctas_per_sm)
@@ -492,7 +514,7 @@ def diffuse_steps(inp, out, r: int, rho: int, k: int, alpha: float = 0.2, map="l
 def block_map(rb: int, order="interleaved", device="cuda", stream=None):
     """Run the device lambda decode for every launch index; returns (bx, by)
     as uint32-valued int32 CUDA tensors (bit patterns, all values < 2^16)."""
-    import torch
+    _bind_torch()
     total = 3 ** rb
     bx = torch.empty(total, dtype=torch.int32, device=device)
     by = torch.empty(total, dtype=torch.int32, device=device)
@@ -516,7 +538,7 @@ class CABatch:
     work list lives in a workspace tensor this object owns."""
 
     def __init__(self, levels, bufs_a, bufs_b, rho=64, autotune=None, stream=None, fuse=1):
-        import torch
+        _bind_torch()
         self.levels = [int(r) for r in levels]
         count = len(self.levels)
         if not (len(bufs_a) == len(bufs_b) == count):
@@ -597,8 +619,8 @@ class Graph:
         self._owner = owner            # keeps the workspace and buffers alive
 
     def launch(self, stream=None):
-        import torch
-        st = torch.cuda.current_stream().cuda_stream if stream is None else (
+        _bind_torch()
+        st = _raw_stream(_current_device()) if stream is None else (
             stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
         _check("sg_graph_launch", int(lib().sg_graph_launch(self.handle, st)))
 
@@ -763,7 +785,7 @@ def compact_size(r: int) -> int:
 
 
 def _compact_check(t, r, dtypes, name):
-    import torch
+    _bind_torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: expected a CUDA tensor (there is no CPU path)")
     if t.dtype not in dtypes:
@@ -773,13 +795,13 @@ def _compact_check(t, r, dtypes, name):
 
 
 def _dtype_id(t):
-    import torch
+    _bind_torch()
     return DTYPES["u8"] if t.dtype == torch.uint8 else DTYPES["f32"]
 
 
 def compact_pack(grid, compact, r: int, rho: int, order=None, stream=None, ctas_per_sm=None):
     """compact <- the gasket cells of the embedded ``grid`` (same dtype)."""
-    import torch
+    _bind_torch()
     _grid_check(grid, r, (torch.uint8, torch.float32), "grid")
     _compact_check(compact, r, (grid.dtype,), "compact")
     with _on_device(grid):
@@ -791,7 +813,7 @@ def compact_pack(grid, compact, r: int, rho: int, order=None, stream=None, ctas_
 
 def compact_unpack(compact, grid, r: int, rho: int, order=None, stream=None, ctas_per_sm=None):
     """The gasket cells of the embedded ``grid`` <- compact (others unchanged)."""
-    import torch
+    _bind_torch()
     _grid_check(grid, r, (torch.uint8, torch.float32), "grid")
     _compact_check(compact, r, (grid.dtype,), "compact")
     with _on_device(grid):
@@ -804,7 +826,7 @@ def compact_unpack(compact, grid, r: int, rho: int, order=None, stream=None, cta
 def compact_map_write(compact, r: int, rho: int, value="hash", value_or_seed=1, order=None,
                       stream=None, ctas_per_sm=None):
     """Map-and-write pass on a compact array (uint8 or float32, 3^r elements)."""
-    import torch
+    _bind_torch()
     _compact_check(compact, r, (torch.uint8, torch.float32), "compact")
     vk = VALUES[value] if isinstance(value, str) else int(value)
     with _on_device(compact):
@@ -818,7 +840,7 @@ def compact_map_write_mapped(host_compact, r: int, rho: int, value="hash", value
                              order=None, stream=None, device=None):
     """Compact write pass straight into a pinned CPU tensor of 3^r elements
     (sg_compact_map_write_mapped).  Returns without synchronising."""
-    import torch
+    _bind_torch()
     if host_compact.is_cuda or not host_compact.is_contiguous() or not host_compact.is_pinned():
         raise TypeError("host_compact: expected a contiguous pinned CPU tensor")
     if host_compact.dtype not in (torch.uint8, torch.float32):
@@ -839,7 +861,7 @@ def compact_map_write_mapped(host_compact, r: int, rho: int, value="hash", value
 
 
 def compact_ca_step(inp, out, r: int, rho: int, order=None, stream=None, ctas_per_sm=None):
-    import torch
+    _bind_torch()
     _compact_check(inp, r, (torch.uint8,), "in")
     _compact_check(out, r, (torch.uint8,), "out")
     with _on_device(inp):
@@ -852,7 +874,7 @@ def compact_ca_step(inp, out, r: int, rho: int, order=None, stream=None, ctas_pe
 def compact_ca_steps(inp, out, r: int, rho: int, k: int, order=None, stream=None,
                      ctas_per_sm=None):
     """k CA steps in one launch on compact states (rho = 64 for k > 1)."""
-    import torch
+    _bind_torch()
     _compact_check(inp, r, (torch.uint8,), "in")
     _compact_check(out, r, (torch.uint8,), "out")
     with _on_device(inp):
@@ -864,7 +886,7 @@ def compact_ca_steps(inp, out, r: int, rho: int, k: int, order=None, stream=None
 
 def compact_diffuse_step(inp, out, r: int, rho: int, alpha: float = 0.2, order=None,
                          stream=None, ctas_per_sm=None):
-    import torch
+    _bind_torch()
     _compact_check(inp, r, (torch.float32,), "in")
     _compact_check(out, r, (torch.float32,), "out")
     with _on_device(inp):
