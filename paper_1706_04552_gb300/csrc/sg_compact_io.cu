@@ -247,7 +247,7 @@ compact_write4_kernel(T *__restrict__ compact, int r, int order, uint32_t total,
             } else {
                 float v[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) v[k] = cv(base[k], koff[i][k]);
+                for (int k = 0; k < 4; ++k) v[k] = cv.float_value(base[k], koff[i][k]);
                 if (e >= 0 && e + 3 < cnt) {
                     *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
                 } else {
