@@ -14,7 +14,7 @@
 //
 // Bound: latency and issue, half and half (the state stays in L2: 14.3 MB read
 // and written at level 15).  Level 15, 16 steps: 180.0 us with dense rows of
-// bits and a 16-cell halo, 24.5 here; level 10: 26.4 and 9.5.
+// bits and a 16-cell halo, 19.5 here; level 10: 26.4 and 8.9.
 #include "sg_compact.cuh"
 #include "sg_words.cuh"
 
@@ -41,19 +41,22 @@ constexpr CellTable make_cell_table()
 }
 __device__ const CellTable kCellTable = make_cell_table();
 
-// 16 bytes at p (16-byte aligned) as 16 bits.  Bytes outside [lo, hi) -- the
-// whole array -- are not read and give 0.
-__device__ __forceinline__ uint32_t piece_bits(const uint8_t *p, const uint8_t *lo,
-                                               const uint8_t *hi)
+__device__ __forceinline__ uint32_t piece_bits(uint4 c)
 {
-    if (p >= lo && p + 16 <= hi) {
-        const uint4 c = __ldg(reinterpret_cast<const uint4 *>(p));
-        return add_nibble(add_nibble(add_nibble(add_nibble(0u, c.w), c.z), c.y), c.x);
-    }
+    return add_nibble(add_nibble(add_nibble(add_nibble(0u, c.w), c.z), c.y), c.x);
+}
+
+// 16 bytes at p as 16 bits where some lie outside [lo, hi), the whole array:
+// those are not read and give 0.
+__device__ __noinline__ uint32_t edge_piece_bits(const uint8_t *p, const uint8_t *lo,
+                                                 const uint8_t *hi)
+{
     uint32_t v = 0u;
-#pragma unroll 1
-    for (int i = 0; i < 16; ++i)
-        if (p + i >= lo && p + i < hi) v |= (uint32_t)(p[i] & 1u) << i;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {         // (unrolled: one memory latency, not sixteen)
+        const uint32_t b = p + i >= lo && p + i < hi ? __ldg(p + i) : 0u;
+        v |= (b & 1u) << i;
+    }
     return v;
 }
 
@@ -64,11 +67,29 @@ __device__ __forceinline__ void run_to_words(uint32_t *s, const uint8_t *run, bo
 {
     const uint32_t off = (uint32_t)((uintptr_t)run & 15u);
     const uint8_t *p = run - off + 96 * warp;
+    const int last = (int)off + kUnit - 96 * warp;    // the run ends here (bytes from p)
     uint32_t b[4] = {0u, 0u, 0u, 0u};                 // 7 pieces: 112 bits from the aligned start
+    // all pieces in the array (every unit but the one with its first or last
+    // tile): the loads go out together
+    if (__all_sync(~0u, !on || (run - off >= lo && run - off + 752 <= hi))) {
+        uint4 c[7];
 #pragma unroll
-    for (int i = 0; i < 7; ++i) {
-        const bool some = on && 96 * warp + 16 * i < (int)off + kUnit;
-        if (some) b[i >> 1] |= piece_bits(p + 16 * i, lo, hi) << (16 * (i & 1));
+        for (int i = 0; i < 7; ++i) {
+            c[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (on && 16 * i < last) c[i] = __ldg(reinterpret_cast<const uint4 *>(p + 16 * i));
+        }
+#pragma unroll
+        for (int i = 0; i < 7; ++i) b[i >> 1] |= piece_bits(c[i]) << (16 * (i & 1));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 7; ++i)
+            if (on && 16 * i < last) {
+                const uint8_t *q = p + 16 * i;
+                const uint32_t v = q >= lo && q + 16 <= hi
+                                       ? piece_bits(__ldg(reinterpret_cast<const uint4 *>(q)))
+                                       : edge_piece_bits(q, lo, hi);
+                b[i >> 1] |= v << (16 * (i & 1));
+            }
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -105,7 +126,7 @@ __device__ __forceinline__ void words_to_run(const uint32_t *s, uint8_t *run, bo
                 *reinterpret_cast<uint4 *>(q) = make_uint4(nibble_bytes(v, 0), nibble_bytes(v, 1),
                                                            nibble_bytes(v, 2), nibble_bytes(v, 3));
             } else {
-#pragma unroll 1
+#pragma unroll 4
                 for (int j = 0; j < 16; ++j)
                     if (e + j >= 0 && e + j < kUnit) q[j] = (uint8_t)((v >> j) & 1u);
             }
@@ -113,7 +134,30 @@ __device__ __forceinline__ void words_to_run(const uint32_t *s, uint8_t *run, bo
     }
 }
 
-__global__ void __launch_bounds__(kWordThreads, kWordCtas)
+// Where the tiles across the corners of unit q lie, as launch indices of the
+// interleaved order (digits finest first: 0 the lower, 1 the upper left, 2 the
+// right third).  At corner A, B, C (digit at = 1, 2, 0) the unit's finest digits
+// that equal `at` are skipped; if the next one is d, the triangle across is the
+// one with d replaced by `at` and the finer digits, down to the tiles, by d.
+// ~0u: none.
+__device__ __forceinline__ uint32_t corner_tile_index(uint32_t q, uint32_t at, int rbu, int l)
+{
+    uint32_t pw = 1u, rest = q, d = at;
+    int j = 0;
+    for (; j < rbu; ++j, pw *= 3u) {
+        const uint32_t n = rest / 3u;
+        d = rest - 3u * n;
+        rest = n;
+        if (d != at) break;
+    }
+    if (j == rbu) return ~0u;
+    const uint32_t per = (uint32_t)pow3i(l);
+    const uint32_t unit = q + (at - d) * (pw - (pw - 1u) / 2u);
+    return unit * per + d * ((per - 1u) / 2u);
+}
+
+template <int CTAS>
+__global__ void __launch_bounds__(kWordThreads, CTAS)
 compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
                      int l, uint32_t units, uint32_t total, int k)
 {
@@ -126,11 +170,26 @@ compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, 
     LambdaLane ll;
     ll.init(lane, rbu, order);
     const uint32_t W = pi_word(order, rbu);
+    // the lane's tile within a unit: base-3 digits 0, 1, 2 of the lane (upper
+    // left, right, lower) are the order's digits 1, 2, 0
+    const uint32_t per = (uint32_t)pow3i(l);
+    uint32_t within = 0u;
+    {
+        uint32_t v = (uint32_t)lane, pw = 1u;
+        for (int j = 0; j < l; ++j, pw *= 3u, v /= 3u) within += (v % 3u + 1u) % 3u * pw;
+    }
+    const uint32_t corner = (uint32_t)lane - per;                 // lanes per .. per + 2
+    const uint32_t at_digit = corner == 0u ? 1u : corner == 1u ? 2u : 0u;
     for (uint32_t q = blockIdx.x; q < units; q += gridDim.x) {
         const uint2 c = decode_tile<kMapLambda>(q, units, rbu, W, ll);
         const WordLane w = unit_lane(nullptr, nullptr, r, l, c.x, c.y, (uint32_t)lane);
         const bool on = w.blocks != 0u;
-        const uint64_t at = (uint64_t)lambda_index(w.x, w.y, r - 6, order) * kUnit;
+        uint32_t tile;
+        if (order == kOrderInterleaved)
+            tile = (uint32_t)lane < per ? q * per + within : corner_tile_index(q, at_digit, rbu, l);
+        else
+            tile = lambda_index(w.x, w.y, r - 6, order);
+        const uint64_t at = (uint64_t)(on ? tile : 0u) * kUnit;
         tr.init(lane);
         run_to_words(st[k & 1], in + at, on, in, in + total, tr, warp, lane);
         words_steps(st, w, t, k, k, false);
@@ -145,16 +204,29 @@ compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, 
 cudaError_t launch_compact_ca_words(int r, int order, const uint8_t *in, uint8_t *out, int k,
                                     cudaStream_t st, const LaunchCfg &cfg)
 {
-    static std::atomic<int> occ{0};
     // unit depth as for the embedded kernel (16 steps, 9 against 27 tiles: level
     // 12, 9.5 and 10.0 us; level 13, 10.3 and 9.9; level 14, 20.4 and 11.8)
     const int l = min(r >= 13 ? 3 : 2, r - 6);
     const uint32_t units = (uint32_t)pow3i(r - 6 - l);
+    int err = 0;
+    const int sms = sm_count(&err);
+    if (err) return (cudaError_t)err;
+    // Units for more than a round of three CTAs an SM: five (48 registers) keep
+    // level 15 to one round (19.5 us against 24.2); below, 63 registers are the
+    // shorter chain (level 10: 8.9 against 9.5).
+    static std::atomic<int> occ3{0}, occ5{0};
     unsigned grid = 1;
-    cudaError_t e = persistent_grid(compact_words_kernel, kWordThreads, 0, units, cfg, &grid, &occ);
-    if (e != cudaSuccess) return e;
-    compact_words_kernel<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units,
-                                                        (uint32_t)pow3i(r), k);
+    if (units > 3u * (uint32_t)sms) {
+        auto k5 = compact_words_kernel<5>;
+        cudaError_t e = persistent_grid(k5, kWordThreads, 0, units, cfg, &grid, &occ5);
+        if (e != cudaSuccess) return e;
+        k5<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units, (uint32_t)pow3i(r), k);
+    } else {
+        auto k3 = compact_words_kernel<3>;
+        cudaError_t e = persistent_grid(k3, kWordThreads, 0, units, cfg, &grid, &occ3);
+        if (e != cudaSuccess) return e;
+        k3<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units, (uint32_t)pow3i(r), k);
+    }
     return cudaGetLastError();
 }
 

@@ -642,8 +642,8 @@ cudaError_t launch_ca_t(int r, int order, const uint8_t *in, uint8_t *out, cudaS
     const uint64_t units = (total + kUnit - 1) / kUnit;
     unsigned grid = 1;
     if constexpr (S == 6) {
-        // on words of 32 tiles from level 14 on (level 14: 9.2 us against 10.7,
-        // level 15: 18.3 against 25.9; level 13: 7.7 against 6.1)
+        // on words of 32 tiles from level 14 on (level 14: 8.5 us against 10.7,
+        // level 15: 14.4 against 25.9; level 13: 7.7 against 6.1)
         if (r >= 14) return launch_compact_ca_words(r, order, in, out, 1, st, cfg);
         auto k = compact_ca_bits_kernel;
         cudaError_t e = persistent_grid(k, kUnitThreads, 0, (units + kUnitWarps - 1) / kUnitWarps,

@@ -164,3 +164,36 @@ def test_compact_runs_shift_to_any_alignment(off_in, off_out):
                         out[off_out + first + j] = (v >> (16 * h + j)) & 1
     assert np.array_equal(out[off_out:off_out + 729], cells)
     assert (out[:off_out] == -1).all() and (out[off_out + 729:] == -1).all()
+
+
+def _corner_tile_index(q, at, rbu, l):
+    pw, rest, d, j = 1, q, at, 0
+    while j < rbu:
+        rest, d = divmod(rest, 3)
+        if d != at:
+            break
+        j, pw = j + 1, 3 * pw
+    if j == rbu:
+        return None
+    per = 3 ** l
+    return (q + (at - d) * (pw - (pw - 1) // 2)) * per + d * ((per - 1) // 2)
+
+
+@pytest.mark.parametrize("rb,l", [(0, 0), (1, 0), (2, 2), (3, 2), (4, 3), (5, 3), (5, 2), (6, 3)])
+def test_corner_tiles_of_a_unit(rb, l):
+    # the tile across each corner of a unit, and the tiles inside it, by the
+    # digits of the interleaved order
+    bx, by = oracle.block_map(rb, oracle.ORDER_INTERLEAVED)
+    place = [(int(x), int(y)) for x, y in zip(bx, by)]
+    index = {p: q for q, p in enumerate(place)}
+    ux, uy = oracle.block_map(rb - l, oracle.ORDER_INTERLEAVED)
+    far, nb = (1 << l) - 1, 1 << rb
+    for q in range(3 ** (rb - l)):
+        ox, oy = int(ux[q]) << l, int(uy[q]) << l
+        for lane in range(3 ** l):
+            x, y = _coords(lane, l)
+            within = sum((lane // 3 ** j % 3 + 1) % 3 * 3 ** j for j in range(l))
+            assert place[q * 3 ** l + within] == (ox + x, oy + y)
+        for c, at, x, y in (("A", 1, ox, oy), ("B", 2, ox + far, oy), ("C", 0, ox, oy + far)):
+            kind, a, b = _neighbour(x, y, nb, c)
+            assert _corner_tile_index(q, at, rb - l, l) == (index[a, b] if kind else None)
