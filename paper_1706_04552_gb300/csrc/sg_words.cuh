@@ -43,7 +43,10 @@ namespace sg {
 constexpr int kWordThreads = 256;
 constexpr int kWordCtas = 3;                    // resident per SM (80 registers a thread)
 constexpr int kTriples = 243;
-constexpr int kPlane = 256;                     // words per plane (A, B, C cells)
+// Words per plane (A, B, C cells): 11 banks apart.  The threads of a warp read
+// their corners in all three planes near their own index; with the planes 256
+// words apart those reads met on the same banks.
+constexpr int kPlane = 267;
 constexpr int kWordZero = 3 * kPlane;           // a word that stays 0
 constexpr int kWordBuf = 3 * kPlane + 8;
 constexpr uint32_t kCornerB = 121, kCornerC = 242;   // digits all 1, all 2 (corner A is 0)
@@ -369,20 +372,29 @@ __device__ __forceinline__ void group_to_words(uint32_t *s, const WordLane &w, u
 {
     const uint8_t *src = w.in + ((u == 2u ? 32ull << w.r : 0ull) + (u == 1u ? 32u : 0u));
     const uint32_t on = w.blocks >> (3u * u);
+    uint32_t *b = s + 81u * u;
+    if constexpr (Q == 0) {
+        // two blocks in flight, then the third: 32 registers of loads, not 48
+        const uint32_t a0 = kChunkTable.at[0][lane], a1 = kChunkTable.at[1][lane];
+        auto words = [&](const uint32_t (&v)[4][4], int j) {
+            const uint32_t x0 = tr(pack_rows<Q>(v, 0)), x1 = tr(pack_rows<Q>(v, 2));
+            if (a0 != kNoWord) b[27 * j + a0] = x0;
+            if (a1 != kNoWord) b[27 * j + a1] = x1;
+        };
+        uint32_t v[2][4][4];
+        load_rows<Q>(v[0], src, w.r, on & 1u);
+        load_rows<Q>(v[1], src + 16, w.r, on & 2u);
+        words(v[0], 0);
+        load_rows<Q>(v[0], src + (16ull << w.r), w.r, on & 4u);
+        words(v[1], 1);
+        words(v[0], 2);
+        return;
+    }
     uint32_t v[3][4][RowGroup<Q>::NIB];
     load_rows<Q>(v[0], src, w.r, on & 1u);
     load_rows<Q>(v[1], src + 16, w.r, on & 2u);
     load_rows<Q>(v[2], src + (16ull << w.r), w.r, on & 4u);
-    uint32_t *b = s + 81u * u;
-    if constexpr (Q == 0) {
-        const uint32_t a0 = kChunkTable.at[0][lane], a1 = kChunkTable.at[1][lane];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const uint32_t x0 = tr(pack_rows<Q>(v[j], 0)), x1 = tr(pack_rows<Q>(v[j], 2));
-            if (a0 != kNoWord) b[27 * j + a0] = x0;
-            if (a1 != kNoWord) b[27 * j + a1] = x1;
-        }
-    } else if constexpr (Q < 3) {
+    if constexpr (Q < 3) {
         const uint32_t a = kChunkTable.at[Q + 1][lane];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
