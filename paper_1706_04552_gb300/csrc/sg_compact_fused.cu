@@ -162,7 +162,7 @@ compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, 
                      int l, uint32_t units, uint32_t total, int k)
 {
     __shared__ uint32_t st[2][kWordBuf];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
     const TripleRefs t = kTripleTable.t[threadIdx.x];
     Transpose tr;

@@ -51,6 +51,14 @@ constexpr int kWordZero = 3 * kPlane;           // a word that stays 0
 constexpr int kWordBuf = 3 * kPlane + 8;
 constexpr uint32_t kCornerB = 121, kCornerC = 242;   // digits all 1, all 2 (corner A is 0)
 
+// The warp's index, by a shuffle: the compiler then knows it for uniform, and
+// the branches on it around shuffles and ballots cost no reconvergence (16 steps
+// at level 11, 7.6 us against 7.2).
+__device__ __forceinline__ int uniform_warp()
+{
+    return __shfl_sync(~0u, (int)(threadIdx.x >> 5), 0);
+}
+
 // Index of the gasket cell (x, y) of a level-`levels` gasket: base-3 digit j
 // is 0, 1 or 2 for the bits (x_j, y_j) = (0,0), (1,0), (0,1).
 __host__ __device__ constexpr uint32_t gasket_digits(uint32_t x, uint32_t y, int levels)
@@ -473,7 +481,7 @@ __device__ __forceinline__ void words_to_group(const uint32_t *s, const WordLane
 // group 0 has 6, groups 1 and 2 have 3, group 3 has 2.
 #define SG_WORD_PIECES(F)                                                        \
     do {                                                                         \
-        const int warp_ = threadIdx.x >> 5;                                      \
+        const int warp_ = uniform_warp();                                        \
         if (warp_ < 3) {                                                         \
             F(0, (uint32_t)warp_);                                               \
         } else if (warp_ < 6) {                                                  \
@@ -500,10 +508,7 @@ __device__ __forceinline__ uint32_t maj3w(uint32_t a, uint32_t b, uint32_t c)
 __device__ __forceinline__ void words_steps(uint32_t (&st)[2][kWordBuf], const WordLane &w,
                                             const TripleRefs &t, int kk, int k, bool mixed)
 {
-    // (the warp's index by a shuffle: the compiler then knows it for uniform, and
-    // the branch around the ballots below costs no reconvergence; 16 steps at
-    // level 11, 7.6 us against 7.2)
-    const int warp = __shfl_sync(~0u, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     // the last warp's lanes pass the corner words between the bits: the bit
     // they take from a corner's B or C cell, or A cell, and their own kinds
     uint32_t fa1 = 0u, fa2 = 0u, fb1 = 0u, fb2 = 0u, fc1 = 0u, fc2 = 0u, ml = 0u, mu = 0u;
