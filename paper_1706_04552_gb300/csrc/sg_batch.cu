@@ -325,17 +325,15 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
                 const bool take = todo && incl <= 32u;
                 todo = todo && !take;
                 const uint32_t excl = incl - tiles;
-                // this lane's gasket: the taken one with excl <= lane < incl
-                int g = -1;
-                uint32_t taken = __ballot_sync(~0u, take);
-                int kmax = 0;
-                while (taken != 0u) {
-                    const int src = __ffs((int)taken) - 1;
-                    taken &= taken - 1u;
-                    const uint32_t e0 = __shfl_sync(~0u, excl, src), e1 = __shfl_sync(~0u, incl, src);
-                    kmax = max(kmax, __shfl_sync(~0u, kk, src));
-                    if (lane >= e0 && lane < e1) g = src;
-                }
+                // this lane's gasket: the first with incl > lane, if it is taken
+                uint32_t lo = 0u;
+#pragma unroll
+                for (uint32_t d = 16u; d > 0u; d >>= 1)
+                    if (__shfl_sync(~0u, incl, (int)(lo + d - 1u)) <= lane) lo += d;
+                const uint32_t end_lo = __shfl_sync(~0u, incl, (int)lo);
+                const int take_lo = __shfl_sync(~0u, (int)take, (int)lo);
+                const int g = end_lo > lane && take_lo ? (int)lo : -1;
+                const int kmax = (int)__reduce_max_sync(~0u, take ? (uint32_t)kk : 0u);
                 const int gs = max(g, 0);
                 const int rg = __shfl_sync(~0u, r, gs), kg = __shfl_sync(~0u, kk, gs);
                 const uint32_t tile = lane - __shfl_sync(~0u, excl, gs);
