@@ -215,11 +215,17 @@ write_sector_kernel(T *__restrict__ grid, int r, int order, uint64_t vs, uint64_
     const uint32_t W = MAP == kMapBBox ? 1u : pi_word(order, rb);
     const uint64_t groups = (nunits + 31) / 32;              // 32 units side by side
 
-    for (uint64_t task = warp0; task < groups * pieces; task += nwarps) {
-        // pieces = 1: the whole units; else the units' piece-th row group
-        const uint64_t gi = pieces == 1u ? task : task / pieces;
-        const uint32_t piece = (uint32_t)(task - gi * pieces);
-        const uint32_t p0 = pieces == 1u ? 0u : piece, p1 = pieces == 1u ? SS::PIECES : piece + 1u;
+    const uint64_t tasks = MAP == kMapBBox ? groups : groups * pieces;
+    for (uint64_t task = warp0; task < tasks; task += nwarps) {
+        // pieces = 1: the whole units; else the units' piece-th row group.  (The
+        // bounding box always walks whole units, over constant bounds: its
+        // warps run for a few lanes each and the unrolled walk is shorter.)
+        const uint64_t gi = MAP == kMapBBox || pieces == 1u ? task : task / pieces;
+        uint32_t p0 = 0u, p1 = SS::PIECES;
+        if (MAP != kMapBBox && pieces != 1u) {
+            p0 = (uint32_t)(task - gi * pieces);
+            p1 = p0 + 1u;
+        }
         const uint64_t unit = gi * 32 + (uint64_t)lane;
         const uint64_t q = unit / PER;
         const uint32_t u = (uint32_t)(unit - q * PER);
