@@ -195,9 +195,10 @@ SG_API sg_status sg_map_write(int r, int rho, sg_map map, sg_dtype dtype, void *
  *            and 0 off the gasket (so in/out can be swapped and stepped
  *            again).  Buffers zero-filled once satisfy both conditions.
  *   map      SG_MAP_LAMBDA or SG_MAP_BBOX (others: SG_EUNSUPPORTED)
- * Each tile is staged in shared memory with its halo; tiles are written
- * whole (off-gasket cells inside a non-empty tile are written as 0).
- * Launches one kernel.
+ * Tiles are written whole, or at least every 32-byte sector of them that holds
+ * gasket cells (its off-gasket cells as 0).  rho names launch geometry, not
+ * results: large gaskets step on 64-tiles whatever rho is.  Launches one
+ * kernel.
  */
 SG_API sg_status sg_ca_step(int r, int rho, sg_map map, const uint8_t *in,
                             uint8_t *out, void *stream);
@@ -261,9 +262,8 @@ SG_API sg_status sg_map_write_mapped(int r, int rho, sg_map map, sg_dtype dtype,
 /*
  * sg_ca_steps / sg_diffuse_steps -- k consecutive steps of sg_ca_step /
  * sg_diffuse_step in one launch: out = step^k(in); `in` is not modified.
- * Every tile is staged in shared memory with a halo at least k cells deep
- * (rounded up to 4, 8 or 16 rows and to whole 16-byte chunks across), the k
- * steps run there, and only the tile is written back, so HBM sees the tile
+ * Every tile is read once with the neighbouring cells that k steps can reach,
+ * stepped k times on the chip, and written back once, so HBM sees the tile
  * bytes about once in and once out per launch rather than per step.  Each
  * cell's arithmetic is that of the single step, so the result equals k
  * calls of the single step.  (The paper fuses nothing; the per-tile lambda
@@ -356,9 +356,8 @@ SG_API sg_status sg_graph_destroy(void *graph);
 
 /* k fused steps of every gasket of the batch in one launch (k = 1 .. SG_FUSE_MAX;
  * k = 1 is sg_batch_ca_step): parity 0 reads buf_a and writes k steps later
- * into buf_b, parity 1 the reverse, as for sg_ca_steps.  A warp takes one
- * work item at a time and runs its tile's k steps bit-sliced in shared
- * memory; results equal k single batch steps. */
+ * into buf_b, parity 1 the reverse, as for sg_ca_steps; results equal k single
+ * batch steps. */
 SG_API sg_status sg_batch_ca_steps(const sg_batch_plan *plan, int parity, int k,
                                    const sg_launch_opts *opts, void *stream);
 

@@ -463,7 +463,7 @@ sg_status sg_compact_ca_steps(int r, int rho, int k, const uint8_t *in, uint8_t 
     if (st != SG_OK) return st;
     if (k == 1) return finish(launch_compact_ca(r, s, cfg.order, in, out, (cudaStream_t)stream, cfg));
     if (rho != 64) return SG_EUNSUPPORTED;
-    return finish(launch_compact_ca_words(r, cfg.order, in, out, k, (cudaStream_t)stream, cfg));
+    return finish(launch_compact_ca_words(r, 6, cfg.order, in, out, k, (cudaStream_t)stream, cfg));
 }
 
 sg_status sg_compact_diffuse_step(int r, int rho, const float *in, float *out, float alpha,

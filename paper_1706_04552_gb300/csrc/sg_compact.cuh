@@ -288,8 +288,10 @@ cudaError_t launch_compact_ca(int r, int s, int order, const uint8_t *in, uint8_
                               cudaStream_t st, const LaunchCfg &cfg);
 cudaError_t launch_compact_diffuse(int r, int s, int order, const float *in, float *out,
                                    float alpha, cudaStream_t st, const LaunchCfg &cfg);
-// k (1 .. SG_FUSE_MAX) CA steps in one launch, rho = 64 (sg_compact_fused.cu).
-cudaError_t launch_compact_ca_words(int r, int order, const uint8_t *in, uint8_t *out, int k,
+// k (1 .. SG_FUSE_MAX) CA steps in one launch on words of 64-tiles, level >= 6:
+// rho = 64 in either order, rho = 16 and 32 in the interleaved order, where the
+// tiles of a 64-tile follow one another (sg_compact_fused.cu).
+cudaError_t launch_compact_ca_words(int r, int s, int order, const uint8_t *in, uint8_t *out, int k,
                                     cudaStream_t st, const LaunchCfg &cfg);
 
 }  // namespace sg

@@ -22,24 +22,36 @@ namespace sg {
 
 namespace {
 
-// Word of the e-th cell of a tile (rows top to bottom, each left to right);
-// the positions past the last cell have none.
+// Word of the e-th element of a 64-tile's run of 729; the positions past the
+// last cell have none.  Tile side 64: rows top to bottom, each left to right.
+// Tile sides 16 and 32 in the interleaved order: the 64-tile is a run of 9 or 3
+// whole tiles, in the order of their digits (finest first: 0 the lower, 1 the
+// upper left, 2 the right third).
 struct CellTable {
     uint16_t at[736];
 };
-constexpr CellTable make_cell_table()
+constexpr CellTable make_cell_table(int s)
 {
     CellTable t{};
+    const uint32_t rho = 1u << s;
     int e = 0;
-    for (uint32_t y = 0; y < 64u; ++y)
-        for (uint32_t x = 0; x < 64u; ++x)
-            if ((x & y) == 0u)
-                t.at[e++] = (uint16_t)(((y & 1u) ? 2u : (x & 1u)) * kPlane +
-                                       gasket_digits(x >> 1, y >> 1, 5));
+    for (uint32_t q = 0; q < (uint32_t)pow3i(6 - s); ++q) {
+        uint32_t x0 = 0, y0 = 0, v = q;
+        for (int j = s; j < 6; ++j, v /= 3u) {
+            x0 |= (v % 3u == 2u ? 1u : 0u) << j;
+            y0 |= (v % 3u == 0u ? 1u : 0u) << j;
+        }
+        for (uint32_t y = y0; y < y0 + rho; ++y)
+            for (uint32_t x = x0; x < x0 + rho; ++x)
+                if ((x & y) == 0u)
+                    t.at[e++] = (uint16_t)(((y & 1u) ? 2u : (x & 1u)) * kPlane +
+                                           gasket_digits(x >> 1, y >> 1, 5));
+    }
     for (; e < 736; ++e) t.at[e] = kNoWord;
     return t;
 }
-__device__ const CellTable kCellTable = make_cell_table();
+__device__ const CellTable kCellTables[3] = {make_cell_table(4), make_cell_table(5),
+                                             make_cell_table(6)};
 
 __device__ __forceinline__ uint32_t piece_bits(uint4 c)
 {
@@ -63,7 +75,8 @@ __device__ __noinline__ uint32_t edge_piece_bits(const uint8_t *p, const uint8_t
 // Cells 96 W .. 96 W + 95 of every lane's tile -> words (warp W).
 __device__ __forceinline__ void run_to_words(uint32_t *s, const uint8_t *run, bool on,
                                              const uint8_t *lo, const uint8_t *hi,
-                                             const Transpose &tr, int warp, int lane)
+                                             const Transpose &tr, const CellTable &ct, int warp,
+                                             int lane)
 {
     const uint32_t off = (uint32_t)((uintptr_t)run & 15u);
     const uint8_t *p = run - off + 96 * warp;
@@ -96,20 +109,21 @@ __device__ __forceinline__ void run_to_words(uint32_t *s, const uint8_t *run, bo
         const int g = 3 * warp + i;
         if (g > 22) break;
         const uint32_t x = tr(__funnelshift_r(b[i], b[i + 1], off));
-        const uint32_t a = kCellTable.at[32 * g + lane];
+        const uint32_t a = ct.at[32 * g + lane];
         if (a != kNoWord) s[a] = x;
     }
 }
 
 // The pieces 6 W .. 6 W + 5 of every own tile's output run.
 __device__ __forceinline__ void words_to_run(const uint32_t *s, uint8_t *run, bool own,
-                                             const Transpose &tr, int warp, int lane)
+                                             const Transpose &tr, const CellTable &ct, int warp,
+                                             int lane)
 {
     uint32_t g[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int e = 96 * warp - 32 + 32 * i + lane;
-        const uint32_t a = e >= 0 && e < 736 ? kCellTable.at[e] : kNoWord;
+        const uint32_t a = e >= 0 && e < 736 ? ct.at[e] : kNoWord;
         g[i] = tr(a != kNoWord ? s[a] : 0u);
     }
     if (!own) return;
@@ -159,8 +173,9 @@ __device__ __forceinline__ uint32_t corner_tile_index(uint32_t q, uint32_t at, i
 template <int CTAS>
 __global__ void __launch_bounds__(kWordThreads, CTAS)
 compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
-                     int l, uint32_t units, uint32_t total, int k)
+                     int l, uint32_t units, uint32_t total, int k, int s)
 {
+    const CellTable &ct = kCellTables[s - 4];
     __shared__ uint32_t st[2][kWordBuf];
     const int warp = uniform_warp(), lane = threadIdx.x & 31;
     if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
@@ -191,17 +206,17 @@ compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, 
             tile = lambda_index(w.x, w.y, r - 6, order);
         const uint64_t at = (uint64_t)(on ? tile : 0u) * kUnit;
         tr.init(lane);
-        run_to_words(st[k & 1], in + at, on, in, in + total, tr, warp, lane);
+        run_to_words(st[k & 1], in + at, on, in, in + total, tr, ct, warp, lane);
         words_steps(st, w, t, k, k, false);
         tr.init(lane);
-        words_to_run(st[0], out + at, w.own, tr, warp, lane);
+        words_to_run(st[0], out + at, w.own, tr, ct, warp, lane);
         __syncthreads();                 // the words are read before the next unit's are written
     }
 }
 
 }  // namespace
 
-cudaError_t launch_compact_ca_words(int r, int order, const uint8_t *in, uint8_t *out, int k,
+cudaError_t launch_compact_ca_words(int r, int s, int order, const uint8_t *in, uint8_t *out, int k,
                                     cudaStream_t st, const LaunchCfg &cfg)
 {
     // unit depth as for the embedded kernel (16 steps, 9 against 27 tiles: level
@@ -220,12 +235,12 @@ cudaError_t launch_compact_ca_words(int r, int order, const uint8_t *in, uint8_t
         auto k5 = compact_words_kernel<5>;
         cudaError_t e = persistent_grid(k5, kWordThreads, 0, units, cfg, &grid, &occ5);
         if (e != cudaSuccess) return e;
-        k5<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units, (uint32_t)pow3i(r), k);
+        k5<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units, (uint32_t)pow3i(r), k, s);
     } else {
         auto k3 = compact_words_kernel<3>;
         cudaError_t e = persistent_grid(k3, kWordThreads, 0, units, cfg, &grid, &occ3);
         if (e != cudaSuccess) return e;
-        k3<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units, (uint32_t)pow3i(r), k);
+        k3<<<grid, kWordThreads, 0, st>>>(in, out, r, order, l, units, (uint32_t)pow3i(r), k, s);
     }
     return cudaGetLastError();
 }

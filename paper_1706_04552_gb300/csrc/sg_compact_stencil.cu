@@ -644,7 +644,7 @@ cudaError_t launch_ca_t(int r, int order, const uint8_t *in, uint8_t *out, cudaS
     if constexpr (S == 6) {
         // on words of 32 tiles from level 14 on (level 14: 8.5 us against 10.7,
         // level 15: 14.4 against 25.9; level 13: 7.7 against 6.1)
-        if (r >= 14) return launch_compact_ca_words(r, order, in, out, 1, st, cfg);
+        if (r >= 14) return launch_compact_ca_words(r, 6, order, in, out, 1, st, cfg);
         auto k = compact_ca_bits_kernel;
         cudaError_t e = persistent_grid(k, kUnitThreads, 0, (units + kUnitWarps - 1) / kUnitWarps,
                                         cfg, &grid, &occ);
@@ -704,6 +704,11 @@ cudaError_t launch_diffuse_t(int r, int order, const float *in, float *out, floa
 cudaError_t launch_compact_ca(int r, int s, int order, const uint8_t *in, uint8_t *out,
                               cudaStream_t st, const LaunchCfg &cfg)
 {
+    // 16- and 32-tiles in the interleaved order on words (us, gathered against
+    // words: rho 16, level 8, 7.9 and 6.5, level 15, 43.6 and 14.3; rho 32, 6.9
+    // and 6.3, 36.4 and 14.3)
+    if ((s == 4 || s == 5) && order == kOrderInterleaved && r >= 6)
+        return launch_compact_ca_words(r, s, order, in, out, 1, st, cfg);
 #define CALL(S) launch_ca_t<S>(r, order, in, out, st, cfg)
     SG_COMPACT_S_SWITCH(s, CALL)
 #undef CALL

@@ -381,10 +381,17 @@ cudaError_t launch_ca(int r, int s, int map, const uint8_t *in, uint8_t *out,
         SG_S_SWITCH(s, CALL)
 #undef CALL
     }
-    // Large gaskets step on words of 32 tiles whatever the tile side (us on
-    // 64-tiles against words: level 13, 5.8 and 6.8; level 14, 13.4 and 10.3;
-    // level 15, 39.2 and 38.0)
-    if (r >= 14 && cfg.store != kStoreTma) return launch_ca_words(r, in, out, 1, st, cfg);
+    // From level 6 on the tile side asked for does not pick the kernel: words of
+    // 32 tiles from level 14 on, a warp per 64-tile at level 13, per 32-tile
+    // below, and cell by cell on 8-tiles up to level 9.  us for tile sides 1, 8,
+    // 16, 32, 64: level 8, 7.9 / 2.4 / 3.0 / 2.8 / 4.0; level 12, 41.9 / 8.3 / 4.6 /
+    // 3.9 / 4.0; level 13, 114 / 18.9 / 8.6 / 7.3 / 5.9 (words 6.8); level 14, 13.4
+    // on 64-tiles, words 10.3; level 15, 39.2 and 38.0.
+    if (r >= 6 && cfg.store != kStoreTma) {
+        if (r >= 14) return launch_ca_words(r, in, out, 1, st, cfg);
+        if (r == 13) return launch_ca_t<6, kMapLambda>(r, in, out, st, cfg);
+        if (s != 3 || r >= 10) return launch_ca_t<5, kMapLambda>(r, in, out, st, cfg);
+    }
 #define CALL(S) launch_ca_t<S, kMapLambda>(r, in, out, st, cfg)
     SG_S_SWITCH(s, CALL)
 #undef CALL

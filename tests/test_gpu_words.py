@@ -125,3 +125,32 @@ def test_single_steps_on_words_match_the_general_path():
     sg.CABatch([7, r], sa, sb, rho=32).step(0)
     assert torch.equal(sb[1], want)
     assert np.array_equal(sb[0].cpu().numpy().reshape(128, 128), oracle.ca_steps(7, _state(7, 1), 1))
+
+
+@pytest.mark.parametrize("r", [6, 9, 10, 12, 13])
+@pytest.mark.parametrize("rho", [1, 8, 16, 64])
+def test_single_step_kernel_is_picked_by_level(r, rho):
+    n = 1 << r
+    a = torch.from_numpy(_state(r, r).ravel()).cuda()
+    want, got = torch.zeros_like(a), torch.zeros_like(a)
+    sg.ca_step(a, want, r, 16, "bbox")
+    sg.ca_step(a, got, r, rho)
+    assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("r,rho,shift_in,shift_out", [
+    (6, 16, 0, 3), (7, 32, 9, 0), (9, 16, 1, 15), (10, 32, 0, 0), (12, 16, 5, 2), (13, 32, 0, 8),
+])
+def test_compact_step_on_smaller_tiles(r, rho, shift_in, shift_out):
+    c = 3 ** r
+    s = rho.bit_length() - 1
+    s0 = _state(r, 70 + r)
+    src = torch.full((c + 64,), 1, dtype=torch.uint8, device="cuda")
+    dst = torch.full((c + 64,), 7, dtype=torch.uint8, device="cuda")
+    a, b = src[shift_in:shift_in + c], dst[shift_out:shift_out + c]
+    a.copy_(torch.from_numpy(oracle.compact_pack(r, s, s0)))
+    sg.compact_ca_step(a, b, r, rho)
+    got = dst.cpu().numpy()
+    assert np.array_equal(got[shift_out:shift_out + c],
+                          oracle.compact_pack(r, s, oracle.ca_steps(r, s0, 1)))
+    assert (got[:shift_out] == 7).all() and (got[shift_out + c:] == 7).all()

@@ -197,3 +197,18 @@ def test_corner_tiles_of_a_unit(rb, l):
         for c, at, x, y in (("A", 1, ox, oy), ("B", 2, ox + far, oy), ("C", 0, ox, oy + far)):
             kind, a, b = _neighbour(x, y, nb, c)
             assert _corner_tile_index(q, at, rb - l, l) == (index[a, b] if kind else None)
+
+
+@pytest.mark.parametrize("s", [4, 5, 6])
+def test_cell_tables_of_smaller_tiles(s):
+    # element e of a 64-tile's run of 729 -> its cell, for tile sides 16, 32, 64
+    rho, cells = 1 << s, []
+    for q in range(3 ** (6 - s)):
+        x0 = y0 = 0
+        for j in range(s, 6):
+            d = q // 3 ** (j - s) % 3
+            x0 |= (d == 2) << j
+            y0 |= (d == 0) << j
+        cells += [(x, y) for y in range(y0, y0 + rho) for x in range(x0, x0 + rho) if x & y == 0]
+    xs, ys = oracle.compact_cells(6, s, oracle.ORDER_INTERLEAVED)
+    assert cells == list(zip(xs.tolist(), ys.tolist()))
