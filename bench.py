@@ -581,7 +581,7 @@ def batched_workload(sg, torch, dev, stream):
     opts = batch.opts
     order = "interleaved" if opts.order == 1 else "rowmajor"
     res = {"gaskets": len(levels), "levels": levels, "steps": steps,
-           "profile": "profiles/batch_ca_bits_l8to12_rho64_k16.md",
+           "profile": "profiles/ca_words_r14_k16.md",
            "cells_per_step": sum(3 ** r for r in levels),
            "tuned": {"rho": batch.rho, "order": order, "ctas_per_sm": opts.ctas_per_sm}}
 
@@ -1082,9 +1082,9 @@ def compare_workloads(sg, torch, dev, stream, w, grid_u8, headline_launch_ms):
                                    "launch_ms": round(statistics.mean(per), 5),
                                    "line_GBps": round(lb / (statistics.mean(per) / 1e3) / 1e9, 1)}
         if mapk == "lambda":
-            _add_traffic(res[f"ca_r{rs}_{mapk}"], f"ca_r{rs}_lambda_rho{rho}", "sg_stencil.cu",
+            _add_traffic(res[f"ca_r{rs}_{mapk}"], f"ca_r{rs}_lambda_rho{rho}", "sg_fused.cu",
                          statistics.mean(per) * 1e3)
-            res[f"ca_r{rs}_{mapk}"]["profile"] = ["profiles/ca_lambda_r15_rho64.md",
+            res[f"ca_r{rs}_{mapk}"]["profile"] = ["profiles/ca_words_r14_k16.md",
                                                   "profiles/stencil_staging_r15.md"]
         del a, b, bufs
     idx, vals = inputs.uniform_sparse(rs, s["diff_seed"])
@@ -1108,8 +1108,8 @@ def compare_workloads(sg, torch, dev, stream, w, grid_u8, headline_launch_ms):
                                           "line_GBps": round(lb / (statistics.mean(per) / 1e3) / 1e9, 1)}
         if mapk == "lambda":
             _add_traffic(res[f"diffusion_r{rs}_{mapk}"], f"diffusion_r{rs}_lambda_rho{rho}",
-                         "sg_stencil.cu", statistics.mean(per) * 1e3)
-            res[f"diffusion_r{rs}_{mapk}"]["profile"] = ["profiles/diffusion_lambda_r14_rho32.md",
+                         "sg_diffuse_tile.cu", statistics.mean(per) * 1e3)
+            res[f"diffusion_r{rs}_{mapk}"]["profile"] = ["profiles/diffuse_tile_r14_k8.md",
                                                          "profiles/stencil_staging_r15.md"]
         del a, b, bufs
     torch.cuda.empty_cache()
@@ -1161,11 +1161,12 @@ def fused_stencils(sg, torch, dev, stream, r, single):
             "us_per_step": round(ms * 1e3 / total, 2), "GCells_s": round(rate, 3),
             "speedup_vs_single_step": round(rate / base, 3) if base else None}
         # DRAM bytes of one launch of k steps, spread over its k steps
-        _add_traffic(out[f"{kind}_r{r}_fused"], f"{kind}_fused_r{r}_rho{rho}_k{k}", "sg_fused.cu",
+        _add_traffic(out[f"{kind}_r{r}_fused"], f"{kind}_fused_r{r}_rho{rho}_k{k}",
+                     "sg_fused.cu" if kind == "ca" else "sg_diffuse_tile.cu",
                      ms * 1e3 / total * k)
-        out[f"{kind}_r{r}_fused"]["profile"] = ("profiles/ca_fused_bits_r15_rho64_k16.md"
+        out[f"{kind}_r{r}_fused"]["profile"] = ("profiles/ca_words_r14_k16.md"
                                                 if kind == "ca" else
-                                                "profiles/diffusion_warp_fused_r14_rho32_k8.md")
+                                                "profiles/diffuse_tile_r14_k8.md")
         del a, bufs
         torch.cuda.empty_cache()
     return out
