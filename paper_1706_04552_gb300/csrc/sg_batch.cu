@@ -7,8 +7,10 @@
 // prefix sum.  A CTA takes a group of consecutive work items, finds each
 // item's gasket by binary search in the prefix sum, decodes the item's tile
 // with lambda at that gasket's level, and runs the CA tile step shared with
-// the single-gasket kernel.  The step sequence can be captured once in a
-// CUDA graph; an autotuner picks rho, the walking order and CTAs per SM.
+// the single-gasket kernel.  Fused steps, and single steps of large batches, run
+// on words of 32 tiles (sg_words.cuh; ca_batch_words_kernel below).  The step
+// sequence can be captured once in a CUDA graph; an autotuner picks rho, the
+// walking order and CTAs per SM.
 //
 // Workspace (caller-owned device memory, sg_batch_workspace_bytes(count)):
 //   uint32 prefix[count + 1]   first work item of gasket i (prefix[count] = total)

@@ -1,6 +1,5 @@
-// sg_bits.cuh -- the bit-sliced B3/S23 CA on one staged tile, shared by the
-// fused single-gasket kernel (sg_fused.cu) and the fused batch kernel
-// (sg_batch.cu).
+// sg_bits.cuh -- the bit-sliced B3/S23 CA on one staged tile, for the bounding
+// box, small gaskets (sg_fused.cu) and small batches (sg_batch.cu).
 #pragma once
 
 #include "sg_stencil.cuh"

@@ -14,7 +14,7 @@
 //
 // Bound: latency and issue, half and half (the state stays in L2: 14.3 MB read
 // and written at level 15).  Level 15, 16 steps: 180.0 us with dense rows of
-// bits and a 16-cell halo, 19.5 here; level 10: 26.4 and 8.9.
+// bits and a 16-cell halo, 18.1 here; level 10: 26.4 and 8.6.
 #include "sg_compact.cuh"
 #include "sg_words.cuh"
 
@@ -220,15 +220,15 @@ cudaError_t launch_compact_ca_words(int r, int s, int order, const uint8_t *in, 
                                     cudaStream_t st, const LaunchCfg &cfg)
 {
     // unit depth as for the embedded kernel (16 steps, 9 against 27 tiles: level
-    // 12, 9.5 and 10.0 us; level 13, 10.3 and 9.9; level 14, 20.4 and 11.8)
+    // 12, 8.5 and 9.3 us; level 13, 9.7 and 9.3; level 14, 15.6 and 11.2)
     const int l = min(r >= 13 ? 3 : 2, r - 6);
     const uint32_t units = (uint32_t)pow3i(r - 6 - l);
     int err = 0;
     const int sms = sm_count(&err);
     if (err) return (cudaError_t)err;
     // Units for more than a round of three CTAs an SM: five (48 registers) keep
-    // level 15 to one round (19.5 us against 24.2); below, 63 registers are the
-    // shorter chain (level 10: 8.9 against 9.5).
+    // level 15 to one round (16 steps, 19.5 us against 23.1); below, more
+    // registers are the shorter chain (level 10: 8.9 against 9.5).
     static std::atomic<int> occ3{0}, occ5{0};
     unsigned grid = 1;
     if (units > 3u * (uint32_t)sms) {

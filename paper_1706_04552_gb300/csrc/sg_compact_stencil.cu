@@ -1,6 +1,11 @@
 // sg_compact_stencil.cu -- the B3/S23 CA step and the diffusion step on
 // compact arrays (layout in sg_compact.cuh).
 //
+// Diffusion at rho >= 16 runs on triples of cells, the CA at rho = 64 on rows of
+// bits and, from level 14 on (rho 16, 32: in the interleaved order always), on
+// words of 32 tiles (sg_compact_fused.cu); all below or there.  The rest runs the
+// gather form:
+//
 // Each warp of a persistent grid takes units of 729 elements (G whole tiles)
 // on its own, with a staging region of its own in shared memory:
 //   1. it decodes the unit's tiles (lambda reduction of Theorem 1) and copies

@@ -518,10 +518,10 @@ diffuse_warp_fused_kernel(const float *__restrict__ in, float *__restrict__ out,
 //
 // Bound: the DRAM pattern of the touched sectors (60 MB in, 60 MB out at level
 // 15), which 32-byte scattered stores sustain at about 3.3 TB/s whatever the
-// kernel; the steps add 0.45 us each.  Level 15, 16 steps: 153.7 us with dense
-// bit rows, 45.0 us here (2 steps: 59.4 and 38.6; level 14, 16 steps: 54.5 and
-// 13.6).  Three CTAs an SM (80 registers, the loads of a unit all in flight)
-// beat five (48 registers, with spills): 45.0 against 47.3 us.
+// kernel; the steps add 0.4 us each.  Level 15, 16 steps: 153.7 us with dense
+// bit rows, 43.5 us here (2 steps: 59.4 and 37.6; level 14, 16 steps: 54.5 and
+// 12.6).  Three CTAs an SM (80 registers) beat four and five (64 and 48, with
+// spills): 43.8 against 47.5 and 44.9 us, 10.5 against 11.6 and 11.9 at level 14.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kWordThreads, kWordCtas)
 ca_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
@@ -546,9 +546,10 @@ cudaError_t launch_ca_words(int r, const uint8_t *in, uint8_t *out, int k, cudaS
                             const LaunchCfg &cfg)
 {
     static std::atomic<int> occ{0};
-    // 27 tiles a unit fill the word (2 and 16 steps at level 13: 6.9 and 9.4 us,
-    // against 7.1 and 10.2 with 9 tiles); below, 9 tiles spread a launch over
-    // more SMs (level 12: 5.6 and 8.1 us against 6.9 and 9.3)
+    // 27 tiles a unit fill the word (2 and 16 steps: level 13, 6.7 and 8.7 us
+    // against 6.7 and 9.1 with 9 tiles; level 14, 10.2 and 12.6 against 13.7 and
+    // 20.2); below, 9 tiles spread a launch over more SMs (level 12: 5.4 and 7.3
+    // us against 6.8 and 8.5)
     const int l = min(r >= 13 ? 3 : 2, max(r - 6, 0));
     const uint32_t units = (uint32_t)pow3i(r > 6 ? r - 6 - l : 0);
     unsigned grid = 1;
@@ -658,18 +659,15 @@ cudaError_t launch_ca_fused(int r, int s, int map, const uint8_t *in, uint8_t *o
     }
     // Small gaskets leave the chip to one wave of warps whichever kernel runs:
     // there a warp per small tile is the shorter chain.  us for 2 / 8 / 16 steps,
-    // dense bit rows on 16-tiles (level 12: 32-tiles) against words: level 9,
-    // 2.8 / 4.2 / 7.1 and 5.2 / 6.2 / 8.1; level 11, 3.4 / 5.4 / 8.9 and 5.4 / 6.7 /
-    // 8.1; level 12, 4.2 / 6.5 / 12.6 and 5.6 / 6.6 / 8.1.
+    // rows of bits on 16-tiles (level 12: 32-tiles) against words: level 9, 3.1 /
+    // 4.4 / 6.9 and 5.2 / 6.0 / 7.0; level 11, 3.6 / 5.3 / 8.9 and 5.5 / 6.1 / 7.1;
+    // level 12, 4.2 / 6.7 / 12.6 and 5.4 / 6.2 / 7.1.
     if (r <= 10 || (r == 11 && k <= 8)) {
         if (k <= 4) return launch_ca_fused_t<4, 4, kMapLambda>(r, in, out, k, st, cfg);
         if (k <= 8) return launch_ca_fused_t<4, 8, kMapLambda>(r, in, out, k, st, cfg);
         return launch_ca_fused_t<4, 16, kMapLambda>(r, in, out, k, st, cfg);
     }
-    if (r == 12 && k <= 8) {
-        if (k <= 4) return launch_ca_fused_t<5, 4, kMapLambda>(r, in, out, k, st, cfg);
-        return launch_ca_fused_t<5, 8, kMapLambda>(r, in, out, k, st, cfg);
-    }
+    if (r == 12 && k <= 4) return launch_ca_fused_t<5, 4, kMapLambda>(r, in, out, k, st, cfg);
     return launch_ca_words(r, in, out, k, st, cfg);
 }
 
