@@ -23,6 +23,7 @@ struct LaunchCfg {
     int ctas_per_sm = 0;
     int order = 1;
     int store = kStoreAuto;
+    bool beside = false;       // batched CA only: may run beside the stream's previous kernel
 };
 
 // Number of SMs of the current device (cached per device).
@@ -34,6 +35,11 @@ namespace sg {
 
 // sg_launch_opts (NULL = defaults) -> LaunchCfg; false on a bad value.
 bool read_launch_opts(const sg_launch_opts *o, LaunchCfg *cfg);
+
+// sg_batch_ca_steps; with `beside` the launch may start while the stream's
+// previous one, also a batched CA launch on other gaskets, still runs.
+sg_status batch_ca_steps(const sg_batch_plan *plan, int parity, int k, const sg_launch_opts *opts,
+                         void *stream, bool beside);
 
 // Record a message for sg_last_error_string().
 void set_last_error_message(const char *msg);

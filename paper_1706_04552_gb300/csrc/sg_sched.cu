@@ -1,7 +1,7 @@
 // sg_sched.cu -- the native core of continuous batching (include/sg_sched.h).
 //
-// Host code only: the kernels are the batch steps of sg_batch.cu, called
-// through the public C ABI (sg_batch_ca_plan_host, sg_batch_ca_steps).  An
+// Host code only: the kernels are the batch steps of sg_batch.cu,
+// planned and launched by sg_batch_ca_plan_host and sg::batch_ca_steps.  An
 // iteration walks the gaskets that hold requests, advances each resident one
 // by min(fuse, steps left in its head request), groups them by the halo that
 // advance needs (1 step; 2..4; 5..8; 9..16), writes every group's
@@ -346,7 +346,9 @@ sg_status sg_sched_step(sg_sched *s, void *stream, sg_sched_result *res)
             sg::set_last_error_message("sg_sched_step: injected launch failure");
             for (int32_t g : m) s->g[g].inject = false;
         } else if (st_launch == SG_OK) {
-            st_launch = sg_batch_ca_steps(&plans[gi], 0, k, opts, stream);
+            // the groups hold different gaskets: the iteration's launches may
+            // overlap one another (not the copy, nor another iteration)
+            st_launch = sg::batch_ca_steps(&plans[gi], 0, k, opts, stream, res->launches > 0);
             if (st_launch == SG_OK) ++res->launches;
         }
         res->active += (int32_t)m.size();
