@@ -87,19 +87,21 @@ __device__ __forceinline__ uint32_t batch_instance(const uint32_t *prefix, uint3
 
 // Two batched launches on different gaskets need not wait for one another: the
 // scheduler's launches of one iteration are chains of 5 to 10 us on a few CTAs
-// each, and a stream would run them one behind the other.  Every batched kernel
-// lets the next launch of the stream start once its own CTAs have (which counts
-// only for one that was launched `beside`), and no CTA ends before the launch in
-// front has: whatever follows the last of them in the stream follows them all.
-// Neither does anything in a launch by itself.
-// (Serving 96 requests on 48 gaskets, 24 launches: 328 us in line, 220 beside.)
+// each, and a stream would run them one behind the other.  With `overlap` (see
+// LaunchCfg) a launch lets the stream's next one start once its own CTAs have,
+// and none of its CTAs ends before the launch in front has: whatever follows the
+// last of them in the stream follows them all.  (Serving 96 requests on 48
+// gaskets, 24 launches: 328 us in line, 220 beside.)  Kernels of their own: the
+// code alone costs a launch by itself 0.2 to 0.4 us, in instruction fetches.
+template <bool OVERLAP>
 __device__ __forceinline__ void let_next_start()
 {
-    asm volatile("griddepcontrol.launch_dependents;");
+    if constexpr (OVERLAP) asm volatile("griddepcontrol.launch_dependents;");
 }
+template <bool OVERLAP>
 __device__ __forceinline__ void end_after_previous()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (OVERLAP) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <typename Kernel, typename... Args>
@@ -115,12 +117,12 @@ cudaError_t launch_kernel(Kernel kernel, unsigned grid, int threads, int smem, c
     c.dynamicSmemBytes = (size_t)smem;
     c.stream = st;
     c.attrs = beside;
-    c.numAttrs = cfg.beside ? 1 : 0;
+    c.numAttrs = cfg.overlap == 2 ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&c, kernel, args...);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int S>
+template <int S, bool OVERLAP>
 __global__ void __launch_bounds__(kStencilThreads)
 ca_batch_kernel(BatchView bv, uint32_t total, int parity, int order)
 {
@@ -128,7 +130,7 @@ ca_batch_kernel(BatchView bv, uint32_t total, int parity, int order)
     __shared__ __align__(16) uint8_t sm[2 * G::TPC * G::TILE];
     __shared__ StencilTile<uint8_t> tiles[2 * G::TPC];
 
-    let_next_start();
+    let_next_start<OVERLAP>();
     LambdaLane ll;
     ll.init(threadIdx.x & 31, 0, order);
     const uint32_t groups = (total + G::TPC - 1) / G::TPC;
@@ -158,12 +160,12 @@ ca_batch_kernel(BatchView bv, uint32_t total, int parity, int order)
         ca_compute_group<S>(buf, slot);
     };
     stencil_pipeline<uint8_t, S>(sm, tiles, groups, decode, compute);
-    end_after_previous();
+    end_after_previous<OVERLAP>();
 }
 
 // One step with one warp per work item (rho = 32, 64): the item's tile is
 // staged and computed by the warp alone, as in the single-gasket kernel.
-template <int S>
+template <int S, bool OVERLAP>
 __global__ void __launch_bounds__(kStencilThreads)
 ca_batch_warp_kernel(BatchView bv, uint32_t total, int parity, int order)
 {
@@ -171,7 +173,7 @@ ca_batch_warp_kernel(BatchView bv, uint32_t total, int parity, int order)
     extern __shared__ __align__(16) unsigned char warp_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *sm = warp_smem + warp * G::TILE;
-    let_next_start();
+    let_next_start<OVERLAP>();
     LambdaLane ll;
     ll.init(lane, 0, order);
     const uint64_t stride = (uint64_t)gridDim.x * kWarpTileWarps;
@@ -191,10 +193,10 @@ ca_batch_warp_kernel(BatchView bv, uint32_t total, int parity, int order)
         for (int k = lane; k < G::CHUNKS; k += 32) ca_chunk<S>(sm, tl, 0, k);
         __syncwarp();                    // the tile is read before the next staging
     }
-    end_after_previous();
+    end_after_previous<OVERLAP>();
 }
 
-template <int S>
+template <int S, bool OVERLAP>
 cudaError_t launch_batch_t(const sg_batch_plan *p, int parity, cudaStream_t st,
                            const LaunchCfg &cfg)
 {
@@ -203,7 +205,7 @@ cudaError_t launch_batch_t(const sg_batch_plan *p, int parity, cudaStream_t st,
     cudaError_t e;
     if constexpr (S >= 5) {
         static std::atomic<uint64_t> attr{0};
-        auto k = ca_batch_warp_kernel<S>;
+        auto k = ca_batch_warp_kernel<S, OVERLAP>;
         constexpr int smem = kWarpTileWarps * StencilGroup<uint8_t, S>::TILE;
         e = dyn_smem_grid(k, smem, ((uint64_t)p->total_tiles + kWarpTileWarps - 1) / kWarpTileWarps,
                           cfg, &grid, &occ, &attr);
@@ -213,7 +215,7 @@ cudaError_t launch_batch_t(const sg_batch_plan *p, int parity, cudaStream_t st,
     } else {
         constexpr int TPC = StencilGroup<uint8_t, S>::TPC;
         const uint64_t groups = (p->total_tiles + TPC - 1) / TPC;
-        auto k = ca_batch_kernel<S>;
+        auto k = ca_batch_kernel<S, OVERLAP>;
         e = persistent_grid(k, kStencilThreads, 0, groups, cfg, &grid, &occ);
         if (e != cudaSuccess) return e;
         return launch_kernel(k, grid, kStencilThreads, 0, st, cfg, view_of(p), p->total_tiles,
@@ -221,13 +223,14 @@ cudaError_t launch_batch_t(const sg_batch_plan *p, int parity, cudaStream_t st,
     }
 }
 
+template <bool OVERLAP>
 cudaError_t launch_batch(const sg_batch_plan *p, int parity, cudaStream_t st,
                          const LaunchCfg &cfg)
 {
     switch (p->rho) {
-    case 16: return launch_batch_t<4>(p, parity, st, cfg);
-    case 32: return launch_batch_t<5>(p, parity, st, cfg);
-    case 64: return launch_batch_t<6>(p, parity, st, cfg);
+    case 16: return launch_batch_t<4, OVERLAP>(p, parity, st, cfg);
+    case 32: return launch_batch_t<5, OVERLAP>(p, parity, st, cfg);
+    case 64: return launch_batch_t<6, OVERLAP>(p, parity, st, cfg);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -235,7 +238,7 @@ cudaError_t launch_batch(const sg_batch_plan *p, int parity, cudaStream_t st,
 // k fused steps of every gasket of a small batch, bit-sliced (sg_bits.cuh): a
 // warp takes one work item at a time, finds its gasket, decodes its tile at
 // that gasket's level and runs the k steps of the tile in shared memory.
-template <int S, int KH>
+template <int S, int KH, bool OVERLAP>
 __global__ void __launch_bounds__(kStencilThreads, 6)
 ca_batch_bits_kernel(BatchView bv, uint32_t total, int parity, int order, int k)
 {
@@ -243,7 +246,7 @@ ca_batch_bits_kernel(BatchView bv, uint32_t total, int parity, int order, int k)
     __shared__ uint32_t sm[B::WARPS][3][B::BUFW];      // two states and the mask, per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t *st0 = sm[warp][0] + 1, *st1 = sm[warp][1] + 1, *mk = sm[warp][2] + 1;
-    let_next_start();
+    let_next_start<OVERLAP>();
     LambdaLane ll;
     ll.init(lane, 0, order);
     const uint64_t stride = (uint64_t)gridDim.x * B::WARPS;
@@ -262,17 +265,17 @@ ca_batch_bits_kernel(BatchView bv, uint32_t total, int parity, int order, int k)
                                reinterpret_cast<uint8_t *>(parity ? pa : pb), r,
                                (int)(c.x << S), (int)(c.y << S), kk, lane);
     }
-    end_after_previous();
+    end_after_previous<OVERLAP>();
 }
 
-template <int S, int KH>
+template <int S, int KH, bool OVERLAP>
 cudaError_t launch_batch_fused_t(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
                                  const LaunchCfg &cfg)
 {
     using B = BitShape<S, KH>;
     static std::atomic<int> occ{0};
     unsigned grid = 1;
-    auto kern = ca_batch_bits_kernel<S, KH>;
+    auto kern = ca_batch_bits_kernel<S, KH, OVERLAP>;
     cudaError_t e = persistent_grid(kern, kStencilThreads, 0,
                                     ((uint64_t)p->total_tiles + B::WARPS - 1) / B::WARPS, cfg,
                                     &grid, &occ);
@@ -307,13 +310,14 @@ __device__ __forceinline__ uint32_t batch_instance_warp(const uint32_t *prefix, 
     return lo;
 }
 
+template <bool OVERLAP>
 __global__ void __launch_bounds__(kWordThreads, kWordCtas)
 ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k, int s, int l,
                       uint32_t window, bool any_small)
 {
     __shared__ uint32_t st[2][kWordBuf];
     const uint32_t lane = threadIdx.x & 31u;
-    let_next_start();
+    let_next_start<OVERLAP>();
     if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
     const TripleRefs t = kTripleTable.t[threadIdx.x];
     LambdaLane ll;
@@ -406,41 +410,58 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
             if (!__all_sync(~0u, in_window)) break;
         }
     }
-    end_after_previous();
+    end_after_previous<OVERLAP>();
 }
 
 // k steps (1 <= k <= SG_FUSE_MAX) of every gasket: one launch.
-cudaError_t launch_batch_k(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
+template <bool OVERLAP>
+cudaError_t launch_batch_overlap(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
                            const LaunchCfg &cfg)
 {
     if (k < 1 || k > SG_FUSE_MAX) return cudaErrorInvalidValue;
     const int s = p->rho == 16 ? 4 : p->rho == 32 ? 5 : 6;
     const uint64_t cells = (uint64_t)p->total_tiles * (uint64_t)pow3i(s);
     // one step: on words from a level-14 gasket's cells on, as for one gasket
-    if (k == 1 && cells < (uint64_t)pow3i(14)) return launch_batch(p, parity, st, cfg);
-    // Few tiles: a warp per 16- or 32-tile is the shorter chain, by the same
-    // lines as for one gasket (launch_ca_fused in sg_fused.cu, in cells)
-    if (s == 4 && (cells <= (uint64_t)pow3i(10) || (cells <= (uint64_t)pow3i(11) && k <= 8))) {
-        if (k <= 4) return launch_batch_fused_t<4, 4>(p, parity, k, st, cfg);
-        if (k <= 8) return launch_batch_fused_t<4, 8>(p, parity, k, st, cfg);
-        return launch_batch_fused_t<4, 16>(p, parity, k, st, cfg);
+    if (k == 1 && cells < (uint64_t)pow3i(14)) return launch_batch<OVERLAP>(p, parity, st, cfg);
+    // Few tiles: a warp per 16- or 32-tile is the shorter chain, up to sizes that
+    // fall as the steps grow (us, rows of bits and words: 16-tiles, 9 steps, 3^11
+    // cells, 7.0 and 7.6; 4 steps, 2 3^11 cells, 6.0 and 7.0; 2 steps, 3^12
+    // cells, 6.2 and 6.6; 32-tiles, 6 steps, 1.5 3^12 cells, 7.9 and 8.7; 4
+    // steps, 2 3^12 cells, 7.6 and 8.5).  Where every gasket is below level 9
+    // the words have one kind of job and win sooner (9 steps on 26 gaskets of
+    // level 8: 7.6 and 7.0).
+    const uint64_t p10 = (uint64_t)pow3i(10), p11 = 3u * p10, p12 = 3u * p11;
+    const uint64_t to10 = p->max_level > (uint32_t)kSmallLevel ? p11 : 2u * p10;
+    if (s == 4 && cells <= (k <= 2 ? p12 : k <= 4 ? 2u * p11 : k <= 8 ? p11 : k <= 11 ? to10 : p10)) {
+        if (k <= 4) return launch_batch_fused_t<4, 4, OVERLAP>(p, parity, k, st, cfg);
+        if (k <= 8) return launch_batch_fused_t<4, 8, OVERLAP>(p, parity, k, st, cfg);
+        return launch_batch_fused_t<4, 16, OVERLAP>(p, parity, k, st, cfg);
     }
-    if (s == 5 && cells <= (uint64_t)pow3i(12) && k <= 8) {
-        if (k <= 4) return launch_batch_fused_t<5, 4>(p, parity, k, st, cfg);
-        return launch_batch_fused_t<5, 8>(p, parity, k, st, cfg);
+    if (s == 5 && cells <= (k <= 4 ? 2u * p12 : k <= 8 ? p12 + p12 / 2u : k <= 11 ? to10 : 0u)) {
+        if (k <= 4) return launch_batch_fused_t<5, 4, OVERLAP>(p, parity, k, st, cfg);
+        if (k <= 8) return launch_batch_fused_t<5, 8, OVERLAP>(p, parity, k, st, cfg);
+        return launch_batch_fused_t<5, 16, OVERLAP>(p, parity, k, st, cfg);
     }
     static std::atomic<int> occ{0};
+    auto kern = ca_batch_words_kernel<OVERLAP>;
     const int l = cells >= (uint64_t)pow3i(13) ? 3 : 2;
     const uint32_t window = (uint32_t)pow3i(l + 6 - s);
     const bool any_small = p->reserved[1] == 0;
     unsigned grid = 1;
-    cudaError_t e = persistent_grid(ca_batch_words_kernel, kWordThreads, 0,
+    cudaError_t e = persistent_grid(kern, kWordThreads, 0,
                                     (any_small ? 2u : 1u) *
                                         (((uint64_t)p->total_tiles + window - 1) / window),
                                     cfg, &grid, &occ);
     if (e != cudaSuccess) return e;
-    return launch_kernel(ca_batch_words_kernel, grid, kWordThreads, 0, st, cfg, view_of(p),
+    return launch_kernel(kern, grid, kWordThreads, 0, st, cfg, view_of(p),
                          p->total_tiles, parity, cfg.order, k, s, l, window, any_small);
+}
+
+cudaError_t launch_batch_k(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
+                           const LaunchCfg &cfg)
+{
+    return cfg.overlap != 0 ? launch_batch_overlap<true>(p, parity, k, st, cfg)
+                            : launch_batch_overlap<false>(p, parity, k, st, cfg);
 }
 
 bool plan_ok(const sg_batch_plan *p)
@@ -604,14 +625,14 @@ sg_status capture_batch(const sg_batch_plan *plan, int steps, int k, int start_p
 }  // namespace
 
 sg_status batch_ca_steps(const sg_batch_plan *plan, int parity, int k, const sg_launch_opts *opts,
-                         void *stream, bool beside)
+                         void *stream, int overlap)
 {
     if (!plan_ok(plan) || (parity != 0 && parity != 1) || k < 1 || k > SG_FUSE_MAX ||
         plan->reserved[0] > k || (k == 1 && plan->reserved[0] > 1))
         return SG_EINVAL;
     LaunchCfg cfg;
     if (!read_launch_opts(opts, &cfg)) return SG_EINVAL;
-    cfg.beside = beside;
+    cfg.overlap = overlap;
     const cudaError_t e = launch_batch_k(plan, parity, k, (cudaStream_t)stream, cfg);
     return e == cudaSuccess ? SG_OK : cuda_fail(e);
 }
@@ -636,7 +657,7 @@ sg_status sg_batch_ca_graph_create_fused(const sg_batch_plan *plan, int steps, i
 sg_status sg_batch_ca_steps(const sg_batch_plan *plan, int parity, int k,
                             const sg_launch_opts *opts, void *stream)
 {
-    return batch_ca_steps(plan, parity, k, opts, stream, false);
+    return batch_ca_steps(plan, parity, k, opts, stream, 0);
 }
 
 sg_status sg_graph_launch(void *graph, void *stream)
@@ -883,6 +904,6 @@ extern "C" sg_status sg_batch_ca_step_noalloc(int count, const int *levels,
     plan.rho = rho;
     plan.total_tiles = (uint32_t)total;
     plan.max_level = (uint32_t)max_level;
-    e = launch_batch(&plan, parity, (cudaStream_t)stream, cfg);
+    e = launch_batch<false>(&plan, parity, (cudaStream_t)stream, cfg);
     return e == cudaSuccess ? SG_OK : cuda_fail(e);
 }

@@ -23,7 +23,9 @@ struct LaunchCfg {
     int ctas_per_sm = 0;
     int order = 1;
     int store = kStoreAuto;
-    bool beside = false;       // batched CA only: may run beside the stream's previous kernel
+    // batched CA only: 1, the next launch may run beside this one; 2, also this
+    // one beside the stream's previous kernel, which was launched with 1 or 2
+    int overlap = 0;
 };
 
 // Number of SMs of the current device (cached per device).
@@ -36,10 +38,10 @@ namespace sg {
 // sg_launch_opts (NULL = defaults) -> LaunchCfg; false on a bad value.
 bool read_launch_opts(const sg_launch_opts *o, LaunchCfg *cfg);
 
-// sg_batch_ca_steps; with `beside` the launch may start while the stream's
-// previous one, also a batched CA launch on other gaskets, still runs.
+// sg_batch_ca_steps with LaunchCfg's overlap: the launches that overlap hold
+// different gaskets.
 sg_status batch_ca_steps(const sg_batch_plan *plan, int parity, int k, const sg_launch_opts *opts,
-                         void *stream, bool beside);
+                         void *stream, int overlap);
 
 // Record a message for sg_last_error_string().
 void set_last_error_message(const char *msg);

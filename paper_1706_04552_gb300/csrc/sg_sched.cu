@@ -348,7 +348,8 @@ sg_status sg_sched_step(sg_sched *s, void *stream, sg_sched_result *res)
         } else if (st_launch == SG_OK) {
             // the groups hold different gaskets: the iteration's launches may
             // overlap one another (not the copy, nor another iteration)
-            st_launch = sg::batch_ca_steps(&plans[gi], 0, k, opts, stream, res->launches > 0);
+            st_launch = sg::batch_ca_steps(&plans[gi], 0, k, opts, stream,
+                                           res->launches > 0 ? 2 : 1);
             if (st_launch == SG_OK) ++res->launches;
         }
         res->active += (int32_t)m.size();

@@ -58,6 +58,22 @@ def test_batch_packs_small_gaskets(rho, levels, k):
         assert np.array_equal(b[i].cpu().numpy().reshape(n, n), want), (i, r)
 
 
+@pytest.mark.parametrize("rho,levels,k", [
+    (16, [12], 2), (16, [10] * 6, 4), (16, [9, 10, 10], 11), (16, [8] * 18, 11), (16, [8] * 19, 9),
+    (32, [11] * 6, 4), (32, [8, 9, 10, 11] * 3, 8), (32, [8, 9, 10, 11] * 3 + [9], 8),
+    (32, [9, 10, 10], 11), (32, [8] * 19, 9), (32, [9], 12),
+])
+def test_batch_around_the_dispatch(rho, levels, k):
+    host = [_state(r, 700 + i) for i, r in enumerate(levels)]
+    a = [torch.from_numpy(h.ravel()).cuda() for h in host]
+    b = [torch.zeros_like(t) for t in a]
+    sg.CABatch(levels, a, b, rho=rho).steps(k, 0)
+    for i, r in enumerate(levels):
+        n = 1 << r
+        assert np.array_equal(b[i].cpu().numpy().reshape(n, n),
+                              oracle.ca_steps(r, host[i], k)), (i, r)
+
+
 def test_scheduler_mixes_step_counts_in_a_word():
     # gaskets that share a word, each with its own step count per iteration
     levels = [6, 7, 6, 8, 9, 6, 7, 10, 6, 8]
