@@ -16,8 +16,8 @@
  *     batched launch serves each class of advances that share a halo size:
  *     1 step, 2..4, 5..8 and 9..16 (each gasket runs its own step count
  *     within its launch: sg_batch_ca_plan_host with steps).  The launches of
- *     an iteration hold different gaskets and may overlap on the device; what
- *     follows the call on the stream follows them all;
+ *     an iteration may overlap on the device unless resident gaskets share
+ *     memory; what follows the call on the stream follows them all;
  *   - the work lists of an iteration are written into page-locked host memory
  *     and reach the device in one asynchronous copy, so an iteration does not
  *     wait for the previous one: the host may prepare iteration i + 1 while
@@ -84,9 +84,10 @@ SG_API sg_status sg_sched_destroy(sg_sched *s);
 
 /*
  * sg_sched_set_buffers -- gasket g's two state buffers (device pointers, n*n
- * bytes each, n = 2^level, 16-byte aligned, distinct and not those of another
- * gasket); `cur` holds its
- * current state.  Both NULL: g is not resident, and its queued requests wait
+ * bytes each, n = 2^level, 16-byte aligned, distinct); `cur` holds its
+ * current state.  Gaskets may share memory (one steps what another has written,
+ * say): an iteration's launches then run one behind the other, the shorter
+ * advances' class first; gaskets of one launch must not.  Both NULL: g is not resident, and its queued requests wait
  * (sg_sched_waiting lists it).  The scheduler swaps the two after each
  * iteration that advances g; sg_sched_gasket reports which one is current.
  */

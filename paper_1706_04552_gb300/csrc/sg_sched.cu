@@ -25,6 +25,7 @@
 #include "sg.h"
 #include "sg_internal.h"
 #include "sg_sched.h"
+#include "sg_spans.h"
 
 namespace {
 
@@ -64,6 +65,11 @@ struct sg_sched {
     bool have_opts = false;
     std::vector<Gasket> g;
     std::vector<int32_t> pending;                  // gaskets with queued requests
+    // The resident gaskets' buffers, unless some share memory (`shared`): the
+    // launches of an iteration then run one behind the other.  `recheck`: buffers
+    // changed while some were shared, so the next iteration looks again.
+    sg::Spans spans;
+    bool shared = false, recheck = false;
     int classes = 1;                               // halo classes in use (by fuse)
     uint64_t slot_bytes = 0;
     unsigned char *img[kSlots] = {nullptr, nullptr};   // page-locked images
@@ -97,6 +103,35 @@ void free_sched(sg_sched *s)
         if (s->dev[j]) cudaFree(s->dev[j]);
     }
     delete s;
+}
+
+// Keep the record of gasket G's buffers (present: they are its current ones).  A
+// failed allocation counts as shared memory: in line is always right.
+void forget_buffers(sg_sched *s, const Gasket &G)
+{
+    if (s->shared) s->recheck = true;
+    if (s->shared || G.cur == nullptr) return;
+    s->spans.remove((uintptr_t)G.cur);
+    s->spans.remove((uintptr_t)G.nxt);
+}
+
+void record_buffers(sg_sched *s, const Gasket &G)
+{
+    if (s->shared || G.cur == nullptr) return;
+    const uint64_t bytes = 1ull << (2 * G.level);
+    try {
+        s->shared = !s->spans.add((uintptr_t)G.cur, bytes) ||
+                    !s->spans.add((uintptr_t)G.nxt, bytes);
+    } catch (...) {
+        s->shared = true;
+    }
+}
+
+void record_all_buffers(sg_sched *s)
+{
+    s->shared = s->recheck = false;
+    s->spans.clear();
+    for (const Gasket &G : s->g) record_buffers(s, G);
 }
 
 // The launch class of an advance of k steps: the halo its fused launch
@@ -174,8 +209,11 @@ sg_status sg_sched_set_buffers(sg_sched *s, int g, uint8_t *cur, uint8_t *nxt)
     if (cur != nullptr &&
         (cur == nxt || ((uintptr_t)cur & 15) != 0 || ((uintptr_t)nxt & 15) != 0))
         return SG_EINVAL;
-    s->g[g].cur = cur;
-    s->g[g].nxt = nxt;
+    Gasket &G = s->g[g];
+    forget_buffers(s, G);
+    G.cur = cur;
+    G.nxt = nxt;
+    record_buffers(s, G);
     return SG_OK;
 }
 
@@ -331,7 +369,12 @@ sg_status sg_sched_step(sg_sched *s, void *stream, sg_sched_result *res)
         s->slot = (j + 1) % kSlots;
     }
 
-    // one launch per group; the host state follows the enqueued work
+    // One launch per group; the host state follows the enqueued work.  The groups
+    // hold different gaskets, so the iteration's launches may overlap one another
+    // (not the copy, nor another iteration) unless gaskets share memory: then one
+    // launch may read or write what another one writes.
+    if (s->recheck) record_all_buffers(s);
+    const bool beside = !s->shared;
     const sg_launch_opts *opts = s->have_opts ? &s->opts : nullptr;
     for (int gi = 0; gi < s->classes; ++gi) {
         const auto &m = s->members[gi];
@@ -346,10 +389,8 @@ sg_status sg_sched_step(sg_sched *s, void *stream, sg_sched_result *res)
             sg::set_last_error_message("sg_sched_step: injected launch failure");
             for (int32_t g : m) s->g[g].inject = false;
         } else if (st_launch == SG_OK) {
-            // the groups hold different gaskets: the iteration's launches may
-            // overlap one another (not the copy, nor another iteration)
             st_launch = sg::batch_ca_steps(&plans[gi], 0, k, opts, stream,
-                                           res->launches > 0 ? 2 : 1);
+                                           !beside ? 0 : res->launches > 0 ? 2 : 1);
             if (st_launch == SG_OK) ++res->launches;
         }
         res->active += (int32_t)m.size();
