@@ -1082,9 +1082,9 @@ def compare_workloads(sg, torch, dev, stream, w, grid_u8, headline_launch_ms):
                                    "launch_ms": round(statistics.mean(per), 5),
                                    "line_GBps": round(lb / (statistics.mean(per) / 1e3) / 1e9, 1)}
         if mapk == "lambda":
-            _add_traffic(res[f"ca_r{rs}_{mapk}"], f"ca_r{rs}_lambda_rho{rho}", "sg_fused.cu",
+            _add_traffic(res[f"ca_r{rs}_{mapk}"], f"ca_r{rs}_lambda_rho{rho}", "sg_stencil.cu",
                          statistics.mean(per) * 1e3)
-            res[f"ca_r{rs}_{mapk}"]["profile"] = ["profiles/ca_words_r14_k16.md",
+            res[f"ca_r{rs}_{mapk}"]["profile"] = ["profiles/ca_lambda_r15_rho64.md",
                                                   "profiles/stencil_staging_r15.md"]
         del a, b, bufs
     idx, vals = inputs.uniform_sparse(rs, s["diff_seed"])

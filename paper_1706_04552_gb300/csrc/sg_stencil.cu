@@ -2,8 +2,8 @@
 // cellular automaton (uint8) and explicit diffusion (float32).
 //
 // Under lambda, diffusion from level 6 on runs in sg_diffuse_tile.cu and the CA
-// from level 14 on in sg_words.cuh; the kernels here serve the bounding box, the
-// smaller gaskets and tensor-copy staging.
+// of level 14 (row-major order: from 14 on) in sg_words.cuh; the kernels here
+// serve the other levels of the CA, the bounding box and tensor-copy staging.
 //
 // The embedded layout keeps (x +- 1, y +- 1) a neighbourhood of the gasket
 // (Section I), so a tile's update needs the tile plus a one-cell halo.  The
@@ -381,15 +381,19 @@ cudaError_t launch_ca(int r, int s, int map, const uint8_t *in, uint8_t *out,
         SG_S_SWITCH(s, CALL)
 #undef CALL
     }
-    // From level 6 on the tile side asked for does not pick the kernel: words of
-    // 32 tiles from level 14 on, a warp per 64-tile at level 13, per 32-tile
-    // below, and cell by cell on 8-tiles up to level 9.  us for tile sides 1, 8,
-    // 16, 32, 64: level 8, 7.9 / 2.4 / 3.0 / 2.8 / 4.0; level 12, 41.9 / 8.3 / 4.6 /
-    // 3.9 / 4.0; level 13, 114 / 18.9 / 8.6 / 7.3 / 5.9 (words 6.8); level 14, 13.4
-    // on 64-tiles, words 10.3; level 15, 39.2 and 38.0.
+    // From level 6 on the tile side asked for does not pick the kernel: a warp per
+    // 32-tile up to level 12 (cell by cell on 8-tiles up to level 9), per 64-tile
+    // above, and words of 32 tiles where they are the faster one.  us, one input
+    // again and again, for tile sides 1, 8, 16, 32, 64: level 8, 7.9 / 2.4 / 3.0 /
+    // 2.8 / 4.0; level 12, 41.9 / 8.3 / 4.6 / 3.9 / 4.0; level 13, 114 / 18.9 / 8.6 /
+    // 7.3 / 5.9 (words 6.8).  64-tiles and words over several inputs in turn: level
+    // 14, 15.3 and 14.1; level 15, 39.5 and 39.3 (other devices: 41.1 and 41.4, 40.4
+    // and 40.9); level 16, 113.5 and 114.1.  In the row-major order level 16 takes
+    // 145 on 64-tiles and 115.5 on words.
     if (r >= 6 && cfg.store != kStoreTma) {
-        if (r >= 14) return launch_ca_words(r, in, out, 1, st, cfg);
-        if (r == 13) return launch_ca_t<6, kMapLambda>(r, in, out, st, cfg);
+        if (r == 14 || (r > 14 && cfg.order != kOrderInterleaved))
+            return launch_ca_words(r, in, out, 1, st, cfg);
+        if (r >= 13) return launch_ca_t<6, kMapLambda>(r, in, out, st, cfg);
         if (s != 3 || r >= 10) return launch_ca_t<5, kMapLambda>(r, in, out, st, cfg);
     }
 #define CALL(S) launch_ca_t<S, kMapLambda>(r, in, out, st, cfg)
