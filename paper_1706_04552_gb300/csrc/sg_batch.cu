@@ -413,6 +413,24 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
     end_after_previous<OVERLAP>();
 }
 
+// Cells from which one step of a batch runs on words.  16- and 32-tiles: a level-14
+// gasket's.  64-tiles are closer (us over several inputs in turn, a warp per
+// 64-tile and words; cells in units of 3^14): where all gaskets have one kind of
+// job and none is above level 10, words win from there on (level 8, 1.0, 19.0 and
+// 16.0; level 10, 1.0, 17.5 and 16.0).  With larger gaskets the units leave a last
+// round nearly empty (level 12, 1.3, 20.4 and 21.0; level 14, 2.0, 28.2 and 28.8;
+// levels 6 to 12 mixed, 1.1, 18.5 and 21.0, 2.1, 32.5 and 33.2, 3.1, 44.0 and
+// 43.2).  Small gaskets of level 9 or 10 between smaller ones leave a window's
+// small job few tiles (levels 6 and 9, 1.1, 20.2 and 22.1, 4.1, 57.2 and 60.7, 6.1,
+// 84.4 and 85.2, 9.0, 123.2 and 121.2).
+uint64_t step_words_from(const sg_batch_plan *p)
+{
+    const uint64_t c14 = (uint64_t)pow3i(14);
+    if (p->rho != 64) return c14;
+    const bool one_kind = p->max_level <= (uint32_t)kSmallLevel || p->reserved[1] != 0;
+    return p->max_level > 10u ? 3u * c14 : one_kind ? c14 : 9u * c14;
+}
+
 // k steps (1 <= k <= SG_FUSE_MAX) of every gasket: one launch.
 template <bool OVERLAP>
 cudaError_t launch_batch_overlap(const sg_batch_plan *p, int parity, int k, cudaStream_t st,
@@ -421,8 +439,7 @@ cudaError_t launch_batch_overlap(const sg_batch_plan *p, int parity, int k, cuda
     if (k < 1 || k > SG_FUSE_MAX) return cudaErrorInvalidValue;
     const int s = p->rho == 16 ? 4 : p->rho == 32 ? 5 : 6;
     const uint64_t cells = (uint64_t)p->total_tiles * (uint64_t)pow3i(s);
-    // one step: on words from a level-14 gasket's cells on, as for one gasket
-    if (k == 1 && cells < (uint64_t)pow3i(14)) return launch_batch<OVERLAP>(p, parity, st, cfg);
+    if (k == 1 && cells < step_words_from(p)) return launch_batch<OVERLAP>(p, parity, st, cfg);
     // Few tiles: a warp per 16- or 32-tile is the shorter chain, up to sizes that
     // fall as the steps grow (us, rows of bits and words: 16-tiles, 9 steps, 3^11
     // cells, 7.0 and 7.6; 4 steps, 2 3^11 cells, 6.0 and 7.0; 2 steps, 3^12

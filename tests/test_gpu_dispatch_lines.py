@@ -33,3 +33,26 @@ def test_one_ca_step_by_level_and_order(r):
                 got.zero_()
                 sg.ca_step(a, got, r, rho, order=order)
                 assert torch.equal(got, want), (shift, rho, order)
+
+
+@pytest.mark.parametrize("levels", [
+    # cells in units of 3^14: small gaskets, below and from 1.0 on; levels 9 and
+    # 10 alone, 1.0; mixed with smaller ones, below and from 9.0 on
+    [8] * 728, [8] * 729, [9, 10] * 62, [10, 8] * 100, [10, 8] * 657,
+    # above level 10, below and from 3.0 on
+    [13, 13, 12, 9, 7], [13] * 8 + [12, 6, 12, 12],
+])
+def test_one_step_of_a_batch_by_cells_and_levels(levels):
+    boards = {r: [_board(r, 31 * r + i) for i in range(2)] for r in set(levels)}
+    want = {}
+    for r, some in boards.items():
+        for i, a in enumerate(some):
+            want[r, i] = torch.zeros_like(a)
+            sg.ca_step(a, want[r, i], r, 16, "bbox")
+    pick = [i % 2 for i in range(len(levels))]
+    a = [boards[r][i].clone() for r, i in zip(levels, pick)]
+    for order in ("interleaved", "rowmajor"):
+        b = [torch.zeros_like(t) for t in a]
+        sg.CABatch(levels, a, b, rho=64).step(0, order=order)
+        for j, (r, i) in enumerate(zip(levels, pick)):
+            assert torch.equal(b[j], want[r, i]), (j, r, order)
