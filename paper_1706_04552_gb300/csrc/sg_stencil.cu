@@ -410,10 +410,14 @@ cudaError_t launch_diffuse(int r, int s, int map, const float *in, float *out,
 #undef CALL
     }
     // A warp per 64-tile with every cell in a register, whatever the tile side;
-    // 16-tiles on small gaskets are the one shorter chain (us, 16-tiles against
-    // it: level 8, 2.6 and 2.9; level 10, 2.8 and 3.1; level 11, 3.2 and 3.0;
-    // level 14, 33.3 and 26.4)
-    if (r >= 6 && cfg.store != kStoreTma && !(s == 4 && r <= 10))
+    // 16-tiles, and 8-tiles at levels 8 and 9, are the shorter chain on small
+    // gaskets (us, the tile side asked for against it; one input again and again:
+    // 16-tiles, level 8, 2.5 and 2.9; level 10, 2.5 and 3.1; 8-tiles, level 7, 2.7
+    // and 2.6; level 8, 2.75 and 2.9; level 10, 2.8 and 2.8; several inputs in
+    // turn: 16-tiles, level 11, 3.2 and 3.5; level 12, 6.1 and 5.6; level 14, 32.9
+    // and 27.3)
+    const bool small = (s == 4 && r <= 11) || (s == 3 && r <= 9 && r >= 8);
+    if (r >= 6 && cfg.store != kStoreTma && !small)
         return launch_diffuse_tile(r, in, out, alpha, 1, st, cfg);
 #define CALL(S) launch_diffuse_t<S, kMapLambda>(r, in, out, alpha, st, cfg)
     SG_S_SWITCH(s, CALL)

@@ -56,3 +56,18 @@ def test_one_step_of_a_batch_by_cells_and_levels(levels):
         sg.CABatch(levels, a, b, rho=64).step(0, order=order)
         for j, (r, i) in enumerate(zip(levels, pick)):
             assert torch.equal(b[j], want[r, i]), (j, r, order)
+
+
+@pytest.mark.parametrize("r,rho", [(7, 8), (8, 8), (9, 8), (10, 8), (10, 16), (11, 16), (12, 16)])
+def test_one_diffusion_step_by_level_and_tile_side(r, rho):
+    # every kernel updates a cell with the same operations in the same order
+    n2 = 1 << (2 * r)
+    idx, val = inputs.uniform_sparse(r, 3 * r)
+    for shift in (0, 4):                         # floats: 16 bytes
+        a, want, got = (torch.zeros(n2 + shift, device="cuda")[shift:] for _ in range(3))
+        a[torch.from_numpy(idx).cuda()] = torch.from_numpy(val).cuda()
+        sg.diffuse_step(a, want, r, 64, 0.2, "bbox")
+        for order in ("interleaved", "rowmajor"):
+            got.zero_()
+            sg.diffuse_step(a, got, r, rho, 0.2, order=order)
+            assert torch.equal(got, want), (shift, order)
