@@ -117,8 +117,12 @@ __device__ __forceinline__ uint32_t stage_unit(T *sv, uint2 *coord, uint8_t *pre
     return cnt;
 }
 
+// Six CTAs an SM, 40 registers: left alone the compiler takes 40 or 32 (and the
+// serial loads that go with 32) as the rest of the file changes.  us at 40 and
+// 32: rho 32, row-major, level 15, 37.5 and 39.1; rho 4, level 10, 23.0 and 23.9;
+// rho 16, row-major, level 15, 48.1 and 50.9 (level 16, 139.7 and 136.9).
 template <int S>
-__global__ void __launch_bounds__(kUnitThreads)
+__global__ void __launch_bounds__(kUnitThreads, 6)
 compact_ca_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
                   uint32_t total)
 {
