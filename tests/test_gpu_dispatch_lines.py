@@ -71,3 +71,41 @@ def test_one_diffusion_step_by_level_and_tile_side(r, rho):
             got.zero_()
             sg.diffuse_step(a, got, r, rho, 0.2, order=order)
             assert torch.equal(got, want), (shift, order)
+
+
+@pytest.mark.parametrize("r,rho,k,order,shift", [
+    (10, 16, 16, "interleaved", 0),          # rows of bits on 16-tiles
+    (10, 64, 16, "rowmajor", 16),
+    (11, 32, 8, "interleaved", 16),          # the last of them
+    (11, 32, 9, "rowmajor", 0),              # words
+    (12, 16, 4, "interleaved", 0),           # rows of bits on 32-tiles
+    (12, 64, 4, "rowmajor", 16),
+    (12, 32, 3, "interleaved", 0),
+    (12, 16, 5, "rowmajor", 0),              # words
+    (12, 32, 5, "interleaved", 16),
+])
+def test_ca_steps_by_level_and_count(r, rho, k, order, shift):
+    n = 1 << r
+    s0 = inputs.ca_seed_grid(r, 0.45, 20 * r + k)
+    a, b = (torch.zeros(n * n + shift, dtype=torch.uint8, device="cuda")[shift:] for _ in range(2))
+    a.copy_(torch.from_numpy(s0.ravel()))
+    sg.ca_steps(a, b, r, rho, k, order=order)
+    assert np.array_equal(b.cpu().numpy().reshape(n, n), oracle.ca_steps(r, s0, k))
+
+
+@pytest.mark.parametrize("rho", [16, 32, 64])
+@pytest.mark.parametrize("levels", [
+    [12, 12, 11, 9, 10, 12],                 # 3^13 cells and more, none below level 9
+    [12, 11, 9, 10, 9],                      # fewer
+    [12, 12, 12, 6, 8],                      # as many, with small ones
+])
+def test_batch_units_with_and_without_small_gaskets(levels, rho):
+    host = [inputs.ca_seed_grid(r, 0.4, 900 + i) for i, r in enumerate(levels)]
+    a = [torch.from_numpy(h.ravel()).cuda() for h in host]
+    for k, order in ((13, "interleaved"), (16, "rowmajor")):
+        b = [torch.zeros_like(t) for t in a]
+        sg.CABatch(levels, a, b, rho=rho).steps(k, 0, order=order)
+        for i, r in enumerate(levels):
+            n = 1 << r
+            assert np.array_equal(b[i].cpu().numpy().reshape(n, n),
+                                  oracle.ca_steps(r, host[i], k)), (i, r, k)
