@@ -531,14 +531,14 @@ ca_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r
     const uint32_t lane = threadIdx.x & 31u;
     if (threadIdx.x < 16) st[threadIdx.x >> 3][kWordZero + (threadIdx.x & 7)] = 0u;
     const TripleRefs t = kTripleTable.t[threadIdx.x];
-    const int rbu = r > 6 ? r - 6 - l : 0;
+    const int rbu = r - 6 - l;
     LambdaLane ll;
     ll.init((int)lane, rbu, order);
     const uint32_t W = pi_word(order, rbu);
     for (uint32_t q = blockIdx.x; q < units; q += gridDim.x) {
         const uint2 c = decode_tile<kMapLambda>(q, units, rbu, W, ll);
         const WordLane w = unit_lane(in, out, r, l, c.x, c.y, lane);
-        words_unit_steps(st, w, t, k, k, r < 6);
+        words_unit_steps(st, w, t, k, k, false);
     }
 }
 
@@ -550,8 +550,8 @@ cudaError_t launch_ca_words(int r, const uint8_t *in, uint8_t *out, int k, cudaS
     // against 6.7 and 9.1 with 9 tiles; level 14, 10.2 and 12.6 against 13.7 and
     // 20.2); below, 9 tiles spread a launch over more SMs (level 12: 5.4 and 7.3
     // us against 6.8 and 8.5)
-    const int l = min(r >= 13 ? 3 : 2, max(r - 6, 0));
-    const uint32_t units = (uint32_t)pow3i(r > 6 ? r - 6 - l : 0);
+    const int l = r >= 13 ? 3 : 2;
+    const uint32_t units = (uint32_t)pow3i(r - 6 - l);
     unsigned grid = 1;
     cudaError_t e = persistent_grid(ca_words_kernel, kWordThreads, 0, units, cfg, &grid, &occ);
     if (e != cudaSuccess) return e;

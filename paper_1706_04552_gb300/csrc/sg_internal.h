@@ -60,7 +60,7 @@ cudaError_t launch_diffuse(int r, int s, int map, const float *in, float *out,
                            float alpha, cudaStream_t st, const LaunchCfg &cfg);
 cudaError_t launch_ca_fused(int r, int s, int map, const uint8_t *in, uint8_t *out, int k,
                             cudaStream_t st, const LaunchCfg &cfg);
-// k (1 .. 16) CA steps under lambda on words of 32 64-tiles (level >= 4).
+// k (1 .. 16) CA steps under lambda on words of 32 64-tiles (level >= 8).
 cudaError_t launch_ca_words(int r, const uint8_t *in, uint8_t *out, int k, cudaStream_t st,
                             const LaunchCfg &cfg);
 // k (1 .. 8) diffusion steps under lambda, one warp per 64-tile (level >= 6).

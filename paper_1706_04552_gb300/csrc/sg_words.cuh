@@ -168,7 +168,7 @@ __device__ __forceinline__ uint32_t tile_blocks(int r)
     return r >= 6 ? 0x1FFu : r == 5 ? 0x7u : 0x1u;
 }
 
-// Lanes of the unit (ux, uy) of a level-r grid: 3^l tiles in digit order, then
+// Lanes of the unit (ux, uy) of a level-r grid (r >= 6 + l): 3^l tiles in digit order, then
 // the tiles at its corners A, B, C.  Of a corner tile only the blocks a
 // 16-step light cone reaches are read: the 16-block at the touching corner,
 // and where that corner is an A, the block past its far end as well (its
@@ -179,7 +179,7 @@ __device__ __forceinline__ WordLane unit_lane(const uint8_t *in, uint8_t *out, i
     const uint32_t nt = (uint32_t)pow3i(l), far = (1u << l) - 1u;
     WordLane w;
     w.r = r;
-    w.nb = r > 6 ? 1u << (r - 6) : 1u;
+    w.nb = 1u << (r - 6);
     w.ox = ux << l;
     w.oy = uy << l;
     w.l = (uint32_t)l;
@@ -192,7 +192,7 @@ __device__ __forceinline__ WordLane unit_lane(const uint8_t *in, uint8_t *out, i
         const uint2 c = gasket_coords(lane, l);
         w.x += c.x;
         w.y += c.y;
-        w.blocks = tile_blocks(r);
+        w.blocks = 0x1FFu;
     } else if (lane < nt + 3u) {
         uint32_t nx = 0, ny = 0, k = 0;
         if (lane == nt) {                      // its corner B, or its C
