@@ -8,7 +8,8 @@ gasket cells written per second (3^16 cells per pass).  The grid (4.3 GB) and
 the sectors one pass touches (181 MB) are both larger than the 129 MB L2, so
 no L2 flush is needed between passes.
 
-Beside the headline the line carries: the roofline of the write kernel
+Beside the headline the run measures (rates and times in the line, everything
+in the file that --report names): the roofline of the write kernel
 (touched 128-byte lines per launch / CUDA-event launch time, against the
 measured HBM copy bandwidth), the bounding-box map on the same workload, the
 float32 grid, the level-15 CA and diffusion steps (single and fused), the
@@ -66,6 +67,9 @@ def parse_args():
     p.add_argument("--quick", action="store_true",
                    help="headline launches only (no clock soak, extras, e2e or CPU "
                         "baseline): the form used under ncu")
+    p.add_argument("--report", default=None, metavar="FILE",
+                   help="also write everything measured, as JSON, to FILE (the printed line "
+                        "holds the rates and times)")
     p.add_argument("--write-sweep", action="store_true",
                    help="the map-and-write sweep instead of the headline: levels 8..16, "
                         "uint8 and float32, rho 8..64, lambda vs bounding box; prints one "
@@ -95,6 +99,44 @@ def parse_args():
                    help="with --quick: run with this L2 fetch granularity (bytes) as the "
                         "context's limit")
     return p.parse_args()
+
+
+# --------------------------------------------------------------------------
+# the printed line: short enough to be read whole from the end of a log
+# --------------------------------------------------------------------------
+_RATES = ("value", "GCells_s", "launch_ms", "us_per_step", "ms", "ms_per_step", "GBps",
+          "dram_frac", "throughput_rps", "gpu_busy_fraction", "latency_ms_p50", "latency_ms_p99",
+          "max_sustained_rps")
+
+
+def _rates(d):
+    """A leg's rates and times, or those of the legs inside it; plain numbers stay."""
+    leg = {k: d[k] for k in _RATES if isinstance(d.get(k), (int, float))}
+    if leg:
+        return leg
+    return {k: _rates(v) if isinstance(v, dict) else v for k, v in d.items()
+            if isinstance(v, (dict, int, float))}
+
+
+def short_line(out):
+    """run_ours' result with the legs beside the headline cut to rates and times."""
+    line = dict(out)
+    for part in ("serving", "e2e_paths"):
+        if part in out:
+            line[part] = _rates(out[part])
+    if "compare" in out:
+        c = dict(out["compare"])
+        sweeps = {}
+        if "level_sweep" in c:
+            sweeps["level_sweep_us"] = {r: [v["lambda_us"], v["bbox_us"]]
+                                        for r, v in c.pop("level_sweep").items()
+                                        if isinstance(v, dict)}
+        if "write_sweep_best" in c:
+            sweeps["write_sweep_best_us"] = {
+                r: [v["lambda_us"], v["bbox_us"]]
+                for r, v in c.pop("write_sweep_best")["best_per_level"].items()}
+        line["compare"] = {**_rates(c), **sweeps}
+    return line
 
 
 # --------------------------------------------------------------------------
@@ -1529,7 +1571,10 @@ def main():
     try:
         out = run_ours(args, grp)
         if grp.rank == 0:
-            print(json.dumps(out))
+            if args.report:
+                with open(args.report, "w") as f:
+                    json.dump(out, f, indent=1)
+            print(json.dumps(short_line(out)))
     finally:
         grp.close()
     return 0
