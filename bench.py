@@ -623,7 +623,7 @@ def batched_workload(sg, torch, dev, stream):
     opts = batch.opts
     order = "interleaved" if opts.order == 1 else "rowmajor"
     res = {"gaskets": len(levels), "levels": levels, "steps": steps,
-           "profile": "profiles/ca_words_r14_k16.md",
+           "profile": "profiles/batch_words_l8to12_rho64_k16.md",
            "cells_per_step": sum(3 ** r for r in levels),
            "tuned": {"rho": batch.rho, "order": order, "ctas_per_sm": opts.ctas_per_sm}}
 
@@ -1151,7 +1151,7 @@ def compare_workloads(sg, torch, dev, stream, w, grid_u8, headline_launch_ms):
         if mapk == "lambda":
             _add_traffic(res[f"diffusion_r{rs}_{mapk}"], f"diffusion_r{rs}_lambda_rho{rho}",
                          "sg_diffuse_tile.cu", statistics.mean(per) * 1e3)
-            res[f"diffusion_r{rs}_{mapk}"]["profile"] = ["profiles/diffuse_tile_r14_k8.md",
+            res[f"diffusion_r{rs}_{mapk}"]["profile"] = ["profiles/diffuse_tile_r14_k1.md",
                                                          "profiles/stencil_staging_r15.md"]
         del a, b, bufs
     torch.cuda.empty_cache()
