@@ -197,8 +197,9 @@ SG_API sg_status sg_map_write(int r, int rho, sg_map map, sg_dtype dtype, void *
  *   map      SG_MAP_LAMBDA or SG_MAP_BBOX (others: SG_EUNSUPPORTED)
  * Tiles are written whole, or at least every 32-byte sector of them that holds
  * gasket cells (its off-gasket cells as 0).  rho names launch geometry, not
- * results: large gaskets step on 64-tiles whatever rho is.  Launches one
- * kernel.
+ * results.  Under SG_MAP_LAMBDA it does not even pick the kernel from level 6 on
+ * (but for 8-tiles up to level 9): the level does, so a sweep of rho there times
+ * one kernel.  Launches one kernel.
  */
 SG_API sg_status sg_ca_step(int r, int rho, sg_map map, const uint8_t *in,
                             uint8_t *out, void *stream);
@@ -216,6 +217,8 @@ SG_API sg_status sg_ca_step(int r, int rho, sg_map map, const uint8_t *in,
  *   alpha    step weight; the update is a convex combination for
  *            0 <= alpha <= 0.25.  Any finite value is accepted.
  *   map      SG_MAP_LAMBDA or SG_MAP_BBOX
+ *   rho      under SG_MAP_LAMBDA from level 6 on, tile sides other than 16 (up to
+ *            level 11) and 8 (levels 8 and 9) run one kernel, on 64-tiles
  * Launches one kernel.
  */
 SG_API sg_status sg_diffuse_step(int r, int rho, sg_map map, const float *in,
@@ -269,8 +272,14 @@ SG_API sg_status sg_map_write_mapped(int r, int rho, sg_map map, sg_dtype dtype,
  * calls of the single step.  (The paper fuses nothing; the per-tile lambda
  * map is that of Theorem 1.)
  *
- *   k        1 .. SG_FUSE_MAX; k = 1 runs the single-step kernel
- *   rho      16, 32 or 64 (other tile sides: SG_EUNSUPPORTED)
+ *   k        1 .. SG_FUSE_MAX; k = 1 runs the single-step kernel.  Diffusion
+ *            under SG_MAP_LAMBDA is fastest per step at 8: 9 to 16 steps run
+ *            another kernel, and two calls of up to 8 are faster than one
+ *            (level 15, 16 steps, rho 32: 166 against 219 us; rho 16: 2400)
+ *   rho      16, 32 or 64 (other tile sides: SG_EUNSUPPORTED).  Under
+ *            SG_MAP_LAMBDA the CA's kernel goes by the level and k, not by rho;
+ *            so does diffusion's up to 8 steps, but for 16-tiles up to level 9
+ *            and 4 steps
  *   in, out, map, alpha, preconditions and postconditions: as for the
  *            single step.
  * Launches one kernel.

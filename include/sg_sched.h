@@ -13,7 +13,7 @@
  *     request advances by min(fuse, steps left in its head request), so a
  *     gasket never steps past a request and every result is the plain
  *     per-gasket step sequence in the order its requests were queued.  One
- *     batched launch serves each class of advances that share a halo size:
+ *     batched launch serves each class of advances:
  *     1 step, 2..4, 5..8 and 9..16 (each gasket runs its own step count
  *     within its launch: sg_batch_ca_plan_host with steps).  The launches of
  *     an iteration may overlap on the device unless resident gaskets share
@@ -57,7 +57,7 @@ typedef struct sg_sched sg_sched;  /* opaque */
  *
  * steps (host array, or NULL) gives every gasket its own step count, 1 ..
  * SG_FUSE_MAX: a launch of the plan with sg_batch_ca_steps(plan, parity, k)
- * then advances gasket i by steps[i] (the halo is sized for k), and requires
+ * then advances gasket i by steps[i] (the launch is sized for k), and requires
  * k >= every steps[i]; the largest is recorded in plan->reserved[0].  Such a
  * plan cannot be captured into a graph, and sg_batch_ca_step (one step) takes
  * it only when every steps[i] is 1.  NULL: every gasket takes the launch's k.

@@ -12,9 +12,10 @@
 // run, and only its first and last pieces, shared with the neighbouring runs,
 // are stored byte by byte.
 //
-// Bound: latency and issue, half and half (the state stays in L2: 14.3 MB read
-// and written at level 15).  Level 15, 16 steps: 180.0 us with dense rows of
-// bits and a 16-cell halo, 18.1 here; level 10: 26.4 and 8.6.
+// Bound: latency and issue, half and half (14.3 MB read and written at level 15).
+// Level 15, 16 steps, dense rows of bits with a 16-cell halo and here: over several
+// inputs in turn 183.4 and 20.3 us, one input again and again (the state stays in
+// the L2) 180.0 and 18.1; level 10, 26.4 and 8.6.
 #include "sg_compact.cuh"
 #include "sg_words.cuh"
 
@@ -219,8 +220,9 @@ compact_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, 
 cudaError_t launch_compact_ca_words(int r, int s, int order, const uint8_t *in, uint8_t *out, int k,
                                     cudaStream_t st, const LaunchCfg &cfg)
 {
-    // unit depth as for the embedded kernel (16 steps, 9 against 27 tiles: level
-    // 12, 8.5 and 9.3 us; level 13, 9.7 and 9.3; level 14, 15.6 and 11.2)
+    // unit depth as for the embedded kernel (one input again and again, 16 steps, 9
+    // against 27 tiles: level 12, 8.5 and 9.3 us; level 13, 9.7 and 9.3; level 14,
+    // 15.6 and 11.2)
     const int l = min(r >= 13 ? 3 : 2, r - 6);
     const uint32_t units = (uint32_t)pow3i(r - 6 - l);
     int err = 0;

@@ -174,7 +174,8 @@ compact_write_kernel(T *__restrict__ compact, int r, int order, uint32_t total, 
 // the multipliers was slower, 41.3 and 43.7 us).  uint8, level 16, with a table
 // load and a byte store per element and here: rho 64, 43.5 and 39.0 us; rho 16,
 // 75.2 and 51.5 (a shuffle per element finds its tile's base); float32, level
-// 15, rho 16: 29.2 and 20.1.
+// 15, rho 16: 29.2 and 20.1.  (Launches back to back; through the call, with three
+// arrays in turn, 45.1 and 41.0 at rho 64.)
 template <typename T, int VK, int S>
 __global__ void __launch_bounds__(kUnitThreads)
 compact_write4_kernel(T *__restrict__ compact, int r, int order, uint32_t total, uint64_t vs)

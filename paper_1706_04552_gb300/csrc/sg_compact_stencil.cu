@@ -25,7 +25,8 @@
 // cells exist here: nothing is spent on the off-gasket 82 % of a 64-tile, and
 // the state of a level-15 CA (14.3 MB) stays in L2.
 //
-// The CA on 64-tiles runs bit-sliced instead (compact_ca_bits_kernel below):
+// The CA on 64-tiles up to level 13 runs bit-sliced instead (compact_ca_bits_kernel
+// below):
 // the gather above spends 9 shared loads per cell and is bound by the L1 /
 // shared-memory pipe, while rows of bits take the rule 64 cells at a time.
 //
@@ -405,10 +406,11 @@ compact_diffuse_kernel(const float *__restrict__ in, float *__restrict__ out, in
 //
 // Bound: HBM (reads and writes 8 bytes a cell, contiguous: 17 us at level 15).
 // Each thread keeps two units' loads in flight while it updates two; one
-// barrier per pair (two publishing buffers).  Level 15, rho 64: 36.2 us with
-// five gathers and a table entry per cell, 20.6 here (one unit at a time 23.6;
-// 7 CTAs an SM with 32 registers and spills 30.6, 5 with 40 registers here);
-// rho 16: 44.7 and 23.4; level 10: 6.9 and 2.2.
+// barrier per pair (two publishing buffers).  Five gathers and a table entry per
+// cell, and here, over several inputs in turn: level 15, rho 64, 37.3 and 21.6 us;
+// rho 16, 45.3 and 24.4; level 14, rho 64, 17.6 and 9.1; level 10 (in the L2), 6.9
+// and 2.2.  One input again and again, level 15, rho 64: 20.6 (one unit at a time
+// 23.6; 7 CTAs an SM with 32 registers and spills 30.6, 5 with 40 registers here).
 // ---------------------------------------------------------------------------
 
 // The tile that touches corner `kind` (0: A, 1: B, 2: C) of tile q in the
@@ -651,8 +653,9 @@ cudaError_t launch_ca_t(int r, int order, const uint8_t *in, uint8_t *out, cudaS
     const uint64_t units = (total + kUnit - 1) / kUnit;
     unsigned grid = 1;
     if constexpr (S == 6) {
-        // on words of 32 tiles from level 14 on (level 14: 8.5 us against 10.7,
-        // level 15: 14.4 against 25.9; level 13: 7.7 against 6.1)
+        // on words of 32 tiles from level 14 on (over several inputs in turn, level
+        // 14, 9.6 us against 11.3; level 15, 16.0 against 27.5; level 16, 38.6
+        // against 75.1; one input again and again, level 13, 7.7 against 6.1)
         if (r >= 14) return launch_compact_ca_words(r, 6, order, in, out, 1, st, cfg);
         auto k = compact_ca_bits_kernel;
         cudaError_t e = persistent_grid(k, kUnitThreads, 0, (units + kUnitWarps - 1) / kUnitWarps,
@@ -714,8 +717,8 @@ cudaError_t launch_compact_ca(int r, int s, int order, const uint8_t *in, uint8_
                               cudaStream_t st, const LaunchCfg &cfg)
 {
     // 16- and 32-tiles in the interleaved order on words (us, gathered against
-    // words: rho 16, level 8, 7.9 and 6.5, level 15, 43.6 and 14.3; rho 32, 6.9
-    // and 6.3, 36.4 and 14.3)
+    // words: rho 16, level 8, 7.9 and 6.5; rho 32, 6.9 and 6.3; over several inputs
+    // in turn, level 15, 46.6 and 16.1; 37.4 and 16.1)
     if ((s == 4 || s == 5) && order == kOrderInterleaved && r >= 6)
         return launch_compact_ca_words(r, s, order, in, out, 1, st, cfg);
 #define CALL(S) launch_ca_t<S>(r, order, in, out, st, cfg)

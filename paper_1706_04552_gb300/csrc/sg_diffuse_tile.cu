@@ -25,12 +25,11 @@
 // tile kernels (a neighbour off the gasket is the 0 the state holds there), so
 // the results are theirs bit for bit, and k steps equal k single steps.
 //
-// Bound: the DRAM pattern of the touched sectors (at level 15, 272 MB read and
-// written at 3.3 TB/s, the rate of every scattered-sector kernel here): 8 steps
-// take 84.0 us and one 82.4, where 32 x 32 units with a frame of halo took 106.5
-// and chunks staged through shared memory 86.6 to 145; level 14: 26.8 and 26.4
-// against 38.7 and 31.3 to 50.  (About 1150 warp instructions per tile and 8
-// steps, 5000 before.)
+// Bound: DRAM's rate for the touched sectors (at level 15, 272 MB read and written
+// at 3.3 TB/s).  Over several inputs in turn, 8 steps take 83.1 us and one 81.8,
+// where 32 x 32 units with a frame of halo took 106.1 and chunks staged through
+// shared memory 85.7 to 145; level 14: 27.9 and 27.4 against 38.6 and 31.1 to 50.
+// (About 1150 warp instructions per tile and 8 steps, 5000 before.)
 #include "sg_stencil.cuh"
 #include "sg_words.cuh"
 

@@ -23,9 +23,9 @@
 // (sg_diffuse_tile.cu).  Here are the bounding-box map and 9 to 16 steps: at tile
 // sides 32 and 64 one warp per 32 x 32 unit with the 9-cell gasket blocks of
 // 4 x 4 cells held in registers (diffuse_warp_fused_kernel, below); at side 16
-// one CTA per tile on float4 chunks (diffuse_fused_kernel).  Either way each cell's result is the single step's,
-// so k fused steps equal k single steps.  HBM moves about the tile bytes once
-// in and once out per launch instead of per step.
+// one CTA per tile on float4 chunks (diffuse_fused_kernel).  Either way each
+// cell's result is the single step's, so k fused steps equal k single steps.  HBM
+// moves about the tile bytes once in and once out per launch instead of per step.
 //
 // The tile coordinate comes from the lambda(omega) decode of Theorem 1 (one
 // warp, redux.sync) or from the bounding-box identity map, as elsewhere.
@@ -516,12 +516,15 @@ diffuse_warp_fused_kernel(const float *__restrict__ in, float *__restrict__ out,
 // (sg_words.cuh), whatever tile side was asked for -- it names launch
 // geometry, not results.  One CTA per unit.
 //
-// Bound: the DRAM pattern of the touched sectors (60 MB in, 60 MB out at level
-// 15), which 32-byte scattered stores sustain at about 3.3 TB/s whatever the
-// kernel; the steps add 0.4 us each.  Level 15, 16 steps: 153.7 us with dense
-// bit rows, 43.5 us here (2 steps: 59.4 and 37.6; level 14, 16 steps: 54.5 and
-// 12.6).  Three CTAs an SM (80 registers) beat four and five (64 and 48, with
-// spills): 43.8 against 47.5 and 44.9 us, 10.5 against 11.6 and 11.9 at level 14.
+// Bound: DRAM's rate for the touched sectors (60 MB in, 60 MB out at level 15)
+// first, then that a CTA's load, steps and store follow one another: 729 units
+// on 456 resident CTAs are 1.6 rounds.  Two steps move 3.1 TB/s of sectors, 16
+// move 2.8, where the warps of diffuse_tile_kernel, each on its own, reach 3.3.
+// Over several inputs in turn, dense bit rows and here: level 15, 16 steps, 151.5
+// and 43.3 us; 2 steps, 59.1 and 38.6; level 14, 16 steps, 56.9 and 16.3 (one
+// input again and again, part of it in the L2: 12.6).  Three CTAs an SM (80
+// registers) beat four and five (64 and 48, with spills): one input again and
+// again, 43.8 against 47.5 and 44.9 us, 10.5 against 11.6 and 11.9 at level 14.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kWordThreads, kWordCtas)
 ca_words_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int r, int order,
@@ -546,7 +549,7 @@ cudaError_t launch_ca_words(int r, const uint8_t *in, uint8_t *out, int k, cudaS
                             const LaunchCfg &cfg)
 {
     static std::atomic<int> occ{0};
-    // 27 tiles a unit fill the word (2 and 16 steps: level 13, 6.7 and 8.7 us
+    // 27 tiles a unit fill the word (one input again and again, 2 and 16 steps: level 13, 6.7 and 8.7 us
     // against 6.7 and 9.1 with 9 tiles; level 14, 10.2 and 12.6 against 13.7 and
     // 20.2); below, 9 tiles spread a launch over more SMs (level 12: 5.4 and 7.3
     // us against 6.8 and 8.5)
@@ -658,7 +661,8 @@ cudaError_t launch_ca_fused(int r, int s, int map, const uint8_t *in, uint8_t *o
 #undef CALL
     }
     // Small gaskets leave the chip to one wave of warps whichever kernel runs:
-    // there a warp per small tile is the shorter chain.  us for 2 / 8 / 16 steps,
+    // there a warp per small tile is the shorter chain.  us for 2 / 8 / 16 steps
+    // (one input again and again; over several in turn level 12, 5 steps, 7.3 and 6.4),
     // rows of bits on 16-tiles (level 12: 32-tiles) against words: level 9, 3.1 /
     // 4.4 / 6.9 and 5.2 / 6.0 / 7.0; level 11, 3.6 / 5.3 / 8.9 and 5.5 / 6.1 / 7.1;
     // level 12, 4.2 / 6.7 / 12.6 and 5.4 / 6.2 / 7.1.
@@ -682,7 +686,9 @@ cudaError_t launch_diffuse_fused(int r, int s, int map, const float *in, float *
     }
     // up to 8 steps: a warp per 64-tile (sg_diffuse_tile.cu), except where a CTA
     // per 16-tile is the shorter chain (us, 2 and 4 steps: level 8, 2.6 and 3.0
-    // against 3.1 and 3.2; level 10, 3.8 and 4.8 against 3.0 and 3.2)
+    // against 3.1 and 3.2; level 10, 3.8 and 4.8 against 3.0 and 3.2).  9 to 16
+    // steps keep the framed units: the cone of more than 8 steps leaves the piece
+    // across a tile's corner.  (Level 15: 16 steps 219 us, two launches of 8, 166.)
     if (k <= 8 && r >= 6 && !(s == 4 && r <= 9 && k <= 4))
         return launch_diffuse_tile(r, in, out, alpha, k, st, cfg);
     if (s == 6) return launch_diffuse_fused_t<6, 16, kMapLambda>(r, in, out, alpha, k, st, cfg);

@@ -3,8 +3,8 @@
 // Host code only: the kernels are the batch steps of sg_batch.cu,
 // planned and launched by sg_batch_ca_plan_host and sg::batch_ca_steps.  An
 // iteration walks the gaskets that hold requests, advances each resident one
-// by min(fuse, steps left in its head request), groups them by the halo that
-// advance needs (1 step; 2..4; 5..8; 9..16), writes every group's
+// by min(fuse, steps left in its head request), groups them by the class of
+// that advance (1 step; 2..4; 5..8; 9..16), writes every group's
 // work list into one page-locked image, copies it to the device in one
 // asynchronous copy and issues one batched launch per group.  The host-side
 // state (queues, which buffer is current) is updated as the work is
@@ -70,7 +70,7 @@ struct sg_sched {
     // changed while some were shared, so the next iteration looks again.
     sg::Spans spans;
     bool shared = false, recheck = false;
-    int classes = 1;                               // halo classes in use (by fuse)
+    int classes = 1;                               // classes of advances in use (by fuse)
     uint64_t slot_bytes = 0;
     unsigned char *img[kSlots] = {nullptr, nullptr};   // page-locked images
     void *dev[kSlots] = {nullptr, nullptr};            // device work lists
@@ -134,9 +134,9 @@ void record_all_buffers(sg_sched *s)
     for (const Gasket &G : s->g) record_buffers(s, G);
 }
 
-// The launch class of an advance of k steps: the halo its fused launch
-// stages (sg_batch_ca_steps sizes it from the launch's k) -- 1 step (the
-// single-step kernel), 2..4, 5..8, 9..16.
+// The launch class of an advance of k steps: 1 (the single-step kernel), 2..4,
+// 5..8, 9..16.  (Rows of bits stage a halo for the class's most steps; words run
+// a launch's most steps, so a class bounds those too.)
 constexpr int kClasses = 4;
 int class_of(int k) { return k <= 1 ? 0 : k <= 4 ? 1 : k <= 8 ? 2 : 3; }
 
@@ -314,7 +314,7 @@ sg_status sg_sched_step(sg_sched *s, void *stream, sg_sched_result *res)
     cudaStream_t st = (cudaStream_t)stream;
 
     // the resident gaskets with requests: each advances by min(fuse, steps
-    // left in its head request), grouped by the halo class of that advance
+    // left in its head request), grouped by the class of that advance
     for (auto &m : s->members) m.clear();
     for (int32_t g : s->pending) {
         Gasket &G = s->g[g];

@@ -387,9 +387,10 @@ cudaError_t launch_ca(int r, int s, int map, const uint8_t *in, uint8_t *out,
     // again and again, for tile sides 1, 8, 16, 32, 64: level 8, 7.9 / 2.4 / 3.0 /
     // 2.8 / 4.0; level 12, 41.9 / 8.3 / 4.6 / 3.9 / 4.0; level 13, 114 / 18.9 / 8.6 /
     // 7.3 / 5.9 (words 6.8).  64-tiles and words over several inputs in turn: level
-    // 14, 15.3 and 14.1; level 15, 39.5 and 39.3 (other devices: 41.1 and 41.4, 40.4
-    // and 40.9); level 16, 113.5 and 114.1.  In the row-major order level 16 takes
-    // 145 on 64-tiles and 115.5 on words.
+    // 14, 15.3 and 13.6; level 15, through the call on three devices, 41.3 and 40.4,
+    // 41.3 and 40.8, 41.5 and 41.9; level 16, 113.6 and 113.1, 114.2 and 114.1.  In
+    // the row-major order level 16 takes 140 to 153 on 64-tiles and 114.5 to 116 on
+    // words.
     if (r >= 6 && cfg.store != kStoreTma) {
         if (r == 14 || (r > 14 && cfg.order != kOrderInterleaved))
             return launch_ca_words(r, in, out, 1, st, cfg);

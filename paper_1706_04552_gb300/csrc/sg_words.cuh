@@ -32,7 +32,8 @@
 //
 // Bound.  A step costs a unit about 320 warp instructions (12 per tile, against
 // 128 for the dense bit rows, which also step a 16-cell halo all round), so a
-// launch is bound by moving the tiles' sectors (figures at the kernels).
+// launch is bound by moving the tiles' sectors and by the chain of load, steps
+// and store within a CTA (figures at the kernels).
 #pragma once
 
 #include "sg_stencil.cuh"
