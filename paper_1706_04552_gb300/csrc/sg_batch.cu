@@ -414,9 +414,10 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
 }
 
 // Cells from which one step of a batch runs on words.  16- and 32-tiles: a level-14
-// gasket's.  64-tiles are closer (us over several inputs in turn, a warp per
-// 64-tile and words; cells in units of 3^14): where all gaskets have one kind of
-// job and none is above level 10, words win from there on (level 8, 1.0, 19.0 and
+// gasket's (32-tiles with small and large gaskets: a third more; levels 8 and 10,
+// 1.06, 21.8 and 22.3, 1.5, 29.4 and 25.6).  64-tiles are closer (us over several
+// inputs in turn, a warp per 64-tile and words; cells in units of 3^14): where all
+// gaskets have one kind of job and none is above level 10, words win from there on (level 8, 1.0, 19.0 and
 // 16.0; level 10, 1.0, 17.5 and 16.0).  With larger gaskets the units leave a last
 // round nearly empty (level 12, 1.3, 20.4 and 21.0; level 14, 2.0, 28.2 and 28.8;
 // levels 6 to 12 mixed, 1.1, 18.5 and 21.0, 2.1, 32.5 and 33.2, 3.1, 44.0 and
@@ -426,9 +427,29 @@ ca_batch_words_kernel(BatchView bv, uint32_t total, int parity, int order, int k
 uint64_t step_words_from(const sg_batch_plan *p)
 {
     const uint64_t c14 = (uint64_t)pow3i(14);
-    if (p->rho != 64) return c14;
     const bool one_kind = p->max_level <= (uint32_t)kSmallLevel || p->reserved[1] != 0;
+    if (p->rho != 64) return p->rho == 16 || one_kind ? c14 : c14 + c14 / 3u;
     return p->max_level > 10u ? 3u * c14 : one_kind ? c14 : 9u * c14;
+}
+
+// CTAs an SM up to which k > 1 steps of 16- and 32-tiles run on rows of bits: a warp
+// per tile is the shorter chain while few of them share an SM, and each further CTA
+// an SM is a jump in time.  us, rows and words, of 160 random batches of levels 6 to
+// 13, several inputs in turn, at this many CTAs an SM (16-tiles: 0.56 x 3^11 cells
+// each, 32-tiles: 1.67 x 3^11).  16-tiles: 2 steps, 6.0, 6.6 and 6.8, 6.7, 7.2 and 6.9;
+// 4 steps, 4.8, 7.0 and 7.3, 5.2, 8.0 and 7.2; 8 steps, 2.8, 7.0 and 7.5, 3.1, 8.6 and
+// 7.7; 9 steps, 1.2, 7.2 and 7.6 (small gaskets alone, 7.2 and 6.8); 16 steps, 1.0,
+// 7.6 and 8.7.  32-tiles: 2 steps, 5.5, 9.7 and 10.3, 6.1, 10.7 and 9.1; 4 steps, 4.0,
+// 7.9 and 8.5, 4.3, 9.1 and 8.5; 6 steps, 2.8, 8.0 and 8.7, 3.4, 9.6 and 8.5; 8 steps,
+// 2.0, 7.2 and 7.7, 2.2, 8.8 and 7.7; 9 steps, 0.6, 7.2 and 7.7 (small gaskets alone,
+// 7.8 and 6.8).  Over these batches the rule is within 0.2 % of the faster kernel on
+// average.
+int rows_ctas(const sg_batch_plan *p, int k)
+{
+    const int alone = p->max_level <= (uint32_t)kSmallLevel ? 1 : 0;
+    if (k <= 1 || p->rho == 64) return 0;
+    if (p->rho == 16) return k <= 2 ? 6 : k <= 4 ? 5 : k <= 8 ? 3 : k <= 11 ? 2 - alone : 1;
+    return k <= 2 ? 6 : k <= 4 ? 4 : k <= 6 ? 3 : k <= 8 ? 2 : k <= 11 ? 1 - alone : 0;
 }
 
 // k steps (1 <= k <= SG_FUSE_MAX) of every gasket: one launch.
@@ -440,24 +461,22 @@ cudaError_t launch_batch_overlap(const sg_batch_plan *p, int parity, int k, cuda
     const int s = p->rho == 16 ? 4 : p->rho == 32 ? 5 : 6;
     const uint64_t cells = (uint64_t)p->total_tiles * (uint64_t)pow3i(s);
     if (k == 1 && cells < step_words_from(p)) return launch_batch<OVERLAP>(p, parity, st, cfg);
-    // Few tiles: a warp per 16- or 32-tile is the shorter chain, up to sizes that
-    // fall as the steps grow (us, rows of bits and words: 16-tiles, 9 steps, 3^11
-    // cells, 7.0 and 7.6; 4 steps, 2 3^11 cells, 6.0 and 7.0; 2 steps, 3^12
-    // cells, 6.2 and 6.6; 32-tiles, 6 steps, 1.5 3^12 cells, 7.9 and 8.7; 4
-    // steps, 2 3^12 cells, 7.6 and 8.5).  Where every gasket is below level 9
-    // the words have one kind of job and win sooner (9 steps on 26 gaskets of
-    // level 8: 7.6 and 7.0).
-    const uint64_t p10 = (uint64_t)pow3i(10), p11 = 3u * p10, p12 = 3u * p11;
-    const uint64_t to10 = p->max_level > (uint32_t)kSmallLevel ? p11 : 2u * p10;
-    if (s == 4 && cells <= (k <= 2 ? p12 : k <= 4 ? 2u * p11 : k <= 8 ? p11 : k <= 11 ? to10 : p10)) {
-        if (k <= 4) return launch_batch_fused_t<4, 4, OVERLAP>(p, parity, k, st, cfg);
-        if (k <= 8) return launch_batch_fused_t<4, 8, OVERLAP>(p, parity, k, st, cfg);
-        return launch_batch_fused_t<4, 16, OVERLAP>(p, parity, k, st, cfg);
-    }
-    if (s == 5 && cells <= (k <= 4 ? 2u * p12 : k <= 8 ? p12 + p12 / 2u : k <= 11 ? to10 : 0u)) {
-        if (k <= 4) return launch_batch_fused_t<5, 4, OVERLAP>(p, parity, k, st, cfg);
-        if (k <= 8) return launch_batch_fused_t<5, 8, OVERLAP>(p, parity, k, st, cfg);
-        return launch_batch_fused_t<5, 16, OVERLAP>(p, parity, k, st, cfg);
+    const int most = rows_ctas(p, k);
+    if (most > 0) {
+        int err = 0;
+        const int sms = sm_count(&err);
+        if (err) return (cudaError_t)err;
+        constexpr uint64_t kWarps = kStencilThreads / 32;
+        if (((uint64_t)p->total_tiles + kWarps - 1) / kWarps <= (uint64_t)most * (uint64_t)sms) {
+            if (s == 4) {
+                if (k <= 4) return launch_batch_fused_t<4, 4, OVERLAP>(p, parity, k, st, cfg);
+                if (k <= 8) return launch_batch_fused_t<4, 8, OVERLAP>(p, parity, k, st, cfg);
+                return launch_batch_fused_t<4, 16, OVERLAP>(p, parity, k, st, cfg);
+            }
+            if (k <= 4) return launch_batch_fused_t<5, 4, OVERLAP>(p, parity, k, st, cfg);
+            if (k <= 8) return launch_batch_fused_t<5, 8, OVERLAP>(p, parity, k, st, cfg);
+            return launch_batch_fused_t<5, 16, OVERLAP>(p, parity, k, st, cfg);
+        }
     }
     static std::atomic<int> occ{0};
     auto kern = ca_batch_words_kernel<OVERLAP>;

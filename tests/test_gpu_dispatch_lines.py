@@ -109,3 +109,33 @@ def test_batch_units_with_and_without_small_gaskets(levels, rho):
             n = 1 << r
             assert np.array_equal(b[i].cpu().numpy().reshape(n, n),
                                   oracle.ca_steps(r, host[i], k)), (i, r, k)
+
+
+@pytest.mark.parametrize("rho,levels,k", [
+    # a CTA an SM is 1216 tiles on 152 SMs: the last batch on rows of bits at each
+    # number of steps, and the first on words
+    (16, [8] * 90, 2), (16, [8] * 91, 2), (16, [8] * 75, 4), (16, [8] * 76, 3),
+    (16, [8] * 45, 8), (16, [9] * 15 + [6], 5), (16, [8] * 15, 9), (16, [8] * 16, 11),
+    (16, [9] * 10, 10), (16, [9] * 10 + [7], 9), (16, [8] * 15, 16), (16, [8, 8, 9, 9, 9, 9, 4], 12),
+    (32, [10] * 30, 2), (32, [10] * 31, 2), (32, [10] * 20, 4), (32, [10] * 20 + [5], 4),
+    (32, [10] * 15, 6), (32, [10] * 15 + [6], 5), (32, [10] * 10, 8), (32, [10] * 10 + [7], 7),
+    (32, [10] * 5, 9), (32, [10] * 5 + [5], 11), (32, [8] * 3, 10), (32, [9, 6], 12),
+])
+def test_batch_steps_by_tiles_and_count(rho, levels, k):
+    boards = {r: [_board(r, 17 * r + i) for i in range(2)] for r in set(levels)}
+    want = {}
+    for r, some in boards.items():
+        for i, a in enumerate(some):
+            want[r, i] = torch.zeros_like(a)
+            if r > 4:
+                sg.ca_steps(a, want[r, i], r, 16, k, "bbox")
+            else:
+                s0 = a.cpu().numpy().reshape(1 << r, 1 << r)
+                want[r, i].copy_(torch.from_numpy(oracle.ca_steps(r, s0, k).ravel()))
+    pick = [i % 2 for i in range(len(levels))]
+    a = [boards[r][i].clone() for r, i in zip(levels, pick)]
+    for order in ("interleaved", "rowmajor"):
+        b = [torch.zeros_like(t) for t in a]
+        sg.CABatch(levels, a, b, rho=rho).steps(k, 0, order=order)
+        for j, (r, i) in enumerate(zip(levels, pick)):
+            assert torch.equal(b[j], want[r, i]), (j, r, order)
