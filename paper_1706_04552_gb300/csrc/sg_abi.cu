@@ -248,6 +248,7 @@ sg_status sg_map_write_mapped(int r, int rho, sg_map map, sg_dtype dtype, void *
     const bool can_stage = rho * elem >= 16 && aligned(grid, 16);
     if ((cfg.store == SG_STORE_STAGED || cfg.store == SG_STORE_FILL) && !can_stage)
         return SG_EUNSUPPORTED;
+    cfg.host = true;
     if (cfg.store == SG_STORE_FILL) cfg.store = kStoreFillPlain;
     // the same choice as on a device grid: 32-byte read-merge-write carries
     // over the link better than staged 16-byte chunks

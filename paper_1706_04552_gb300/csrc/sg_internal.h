@@ -23,6 +23,7 @@ struct LaunchCfg {
     int ctas_per_sm = 0;
     int order = 1;
     int store = kStoreAuto;
+    bool host = false;           // the write pass's grid lies in host memory
     // batched CA only: 1, the next launch may run beside this one; 2, also this
     // one beside the stream's previous kernel, which was launched with 1 or 2
     int overlap = 0;

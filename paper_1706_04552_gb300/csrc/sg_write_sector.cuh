@@ -274,9 +274,16 @@ cudaError_t launch_write_sector(int r, T *grid, uint64_t vs, uint64_t ntiles, cu
         // 16, 351 and 242; uint8, level 11, 16.9 and 5.2, level 15, 35.7 and
         // 35.3).  Only the uint8 grid of level 16 (5536 groups) keeps whole
         // units, 114 against 121, and the bounding box, where most of a
-        // group's units are empty.
-        const uint32_t pieces =
-            M != kMapBBox && (sizeof(T) == 4 || groups <= 2048) ? SS::PIECES : 1u;
+        // group's units are empty.  Across the host link the chain of a whole
+        // unit no longer counts once the launch has some hundred groups, and a
+        // lane's requests one after the other do (merge, whole and apart: uint8,
+        // level 13, 79 and 79, level 14, 210 and 224; float32, rho 64, level
+        // 11, 39 and 24, level 12, 59 and 65; masked, 66 and 62, 173 and 184);
+        // with 16-row units and in the write-only form apart stays ahead.
+        bool whole = M == kMapBBox || (sizeof(T) == 1 && groups > 2048);
+        if (cfg.host && (cfg.store == kStoreMerge || cfg.store == kStoreMasked) && SS::US == 32)
+            whole = whole || groups > (sizeof(T) == 1 ? 256u : 32u);
+        const uint32_t pieces = whole ? 1u : SS::PIECES;
         const uint64_t tasks = groups * pieces;
         const uint64_t units = (tasks + kSectorThreads / 32 - 1) / (kSectorThreads / 32);
         unsigned grid_ctas = 1;

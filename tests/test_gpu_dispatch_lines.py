@@ -139,3 +139,25 @@ def test_batch_steps_by_tiles_and_count(rho, levels, k):
         sg.CABatch(levels, a, b, rho=rho).steps(k, 0, order=order)
         for j, (r, i) in enumerate(zip(levels, pick)):
             assert torch.equal(b[j], want[r, i]), (j, r, order)
+
+
+@pytest.mark.parametrize("dtype,r,rho", [
+    (torch.uint8, 13, 64), (torch.uint8, 14, 32), (torch.float32, 10, 16), (torch.float32, 11, 64),
+    (torch.float32, 12, 32), (torch.float32, 12, 16),
+])
+@pytest.mark.parametrize("store", ["merge", "masked", "sector"])
+def test_grids_in_host_memory_by_size(dtype, r, rho, store):
+    # row groups apart or whole units; the device grid takes the first at these sizes
+    n2 = 1 << (2 * r)
+    if store == "sector":
+        start = torch.zeros(n2, dtype=dtype)
+    elif dtype == torch.uint8:
+        start = torch.arange(n2, dtype=torch.int32).remainder_(251).to(dtype)
+    else:
+        start = torch.arange(n2, dtype=torch.float32).remainder_(1009.0)
+    host = start.clone().pin_memory()
+    sg.map_write_mapped(host, r, rho, "lambda", "hash", 5, store=store)
+    dev = start.cuda()
+    sg.map_write(dev, r, rho, "lambda", "hash", 5, store="scatter")
+    torch.cuda.synchronize()
+    assert torch.equal(host, dev.cpu())
